@@ -59,6 +59,7 @@ struct RunEvents {
 
 struct mcpt_ctx {
     int device = 0;
+    int sms = 0;                     // SMs of the device
     cudaStream_t stream = nullptr;
     bool own_stream = false;
     mcpt_precision prec = MCPT_FP64;
@@ -110,6 +111,8 @@ struct mcpt_ctx {
 
     void* dH = nullptr;              // first-half result of one wave (shared by every plan)
     size_t capH = 0;
+    void* dFc = nullptr;             // FP32C: tile counter and per-CTA slots of the first half (shared)
+    size_t capFc = 0;
     void* dVT = nullptr;             // coupling: every dimer's (ia|jb) and T = vD
     size_t capVT = 0;
     void* dCoup = nullptr;           // coupling tables: tiles, per-dimer info, monomer sizes, R offsets
@@ -171,6 +174,8 @@ struct mcpt_ctx {
         double* dPart = nullptr;           // their FP64 partial sums
         size_t capPart = 0;
         std::vector<Wave> waves;
+        int fc_slots = 0;                  // FP32C: scratch slots of the first half (0: the kernel without)
+        size_t fc_slot_bytes = 0;
         double alg_bytes = 0, alg_flops = 0, alg_flops_half = 0;
         int nfold = 0;                     // split dimers whose block results are folded
         bool coupling = false;             // the plan stores (ia|jb), T and forms R
@@ -427,6 +432,7 @@ mcpt_status mcpt_create(mcpt_handle* out, const mcpt_options* opt)
     mcpt_ctx* h = new (std::nothrow) mcpt_ctx;
     if (!h) return fail(nullptr, MCPT_ENOMEM, "mcpt_create: out of host memory");
     h->device = o.device;
+    h->sms = prop.multiProcessorCount;
     h->prec = o.precision;
     h->validate = o.validate;
     h->wave_bytes = o.wave_bytes ? o.wave_bytes : ((size_t)1 << 30);
@@ -958,6 +964,24 @@ static mcpt_status build_plan(mcpt_handle h, mcpt_ctx::Plan& P, int first, int c
     size_t wave_h = 0, max_wave_h = 0;
     int wbeg = 0;
     double alg_bytes = 0.0, alg_flops = 0.0, alg_flops_half = 0.0;
+    // FP32C: a quarter of the run's scratch for the first half's slots, one
+    // per resident CTA.  With room for fewer than one slot per SM, or with a
+    // memory cap (whose every byte may be wanted for integrals added later),
+    // the kernel that needs no slots runs and H has all of the scratch.
+    P.fc_slots = 0;
+    P.fc_slot_bytes = 0;
+    size_t wave_cap = h->wave_bytes;
+    if (prec == MCPT_FP32C && !h->mem_cap) {
+        for (int d = first; d < first + count; d++)
+            P.fc_slot_bytes = std::max(P.fc_slot_bytes, fp32c_slot_bytes(h->mons[h->dims[d].X].nao,
+                                                                         h->mons[h->dims[d].Y].nocc));
+        const size_t fit = std::min<size_t>((size_t)kFp32cSlotsPerSM * h->sms,
+                                            h->wave_bytes / 4 / P.fc_slot_bytes);
+        if (fit >= (size_t)h->sms) {
+            P.fc_slots = (int)fit;
+            wave_cap -= fit * P.fc_slot_bytes;
+        }
+    }
     for (int k = 0; k < count; k++) {
         const int d = first + k;
         const DimerRec& r = h->dims[d];
@@ -1001,7 +1025,7 @@ static mcpt_status build_plan(mcpt_handle h, mcpt_ctx::Plan& P, int first, int c
                 const size_t hb = hbytes_for(prec, dd.nX, dd.nY, dd.oX, dd.oY);
                 const size_t elem = fp64_data(prec) ? 8 : 4;
                 const int kk = (int)P.hDesc.size();
-                if (kk > wbeg && (wave_h + hb > h->wave_bytes || kk - wbeg >= 65535)) {
+                if (kk > wbeg && (wave_h + hb > wave_cap || kk - wbeg >= 65535)) {
                     waves.emplace_back(wbeg, kk);
                     max_wave_h = std::max(max_wave_h, wave_h);
                     wbeg = kk;
@@ -1025,6 +1049,11 @@ static mcpt_status build_plan(mcpt_handle h, mcpt_ctx::Plan& P, int first, int c
     if (st) return st;
     if ((st = ensure(h, &P.dDesc, &P.capDesc, ndesc * sizeof(DimerDesc)))) return st;
     if ((st = ensure_shared(h, &h->dH, &h->capH, max_wave_h))) return st;
+    if (P.fc_slots &&
+        ensure_shared(h, &h->dFc, &h->capFc, kFp32cCounterBytes + P.fc_slots * P.fc_slot_bytes) != MCPT_OK) {
+        h->err.clear();
+        P.fc_slots = 0;                        // no room on the device: the kernel without slots
+    }
     if (!fold.empty() && (st = ensure(h, &P.dFold, &P.capFold, fold.size() * sizeof(int)))) return st;
     // per-dimer results, then the results of split dimers' blocks (kept across
     // plans: a larger array copies the dimers' results over)
@@ -1269,7 +1298,8 @@ static mcpt_status enqueue_run(mcpt_handle h, const mcpt_ctx::Plan& P, const std
             CK(h, launch_half_fp64(wd, wv.nd, wv.max_rows, wv.max_occ, h->dC, static_cast<double*>(h->dH), h->stream));
             break;
         case MCPT_FP32C:
-            CK(h, launch_half_fp32c(wd, wv.nd, wv.max_rows, wv.max_occ, h->dCf, static_cast<float*>(h->dH), h->stream));
+            CK(h, launch_half_fp32c(wd, wv.nd, wv.max_rows, wv.max_occ, h->dCf, static_cast<float*>(h->dH), h->dFc,
+                                    P.fc_slots, P.fc_slot_bytes, h->stream));
             break;
         case MCPT_TF32:
         case MCPT_BF16X3:
@@ -1964,6 +1994,7 @@ void mcpt_destroy(mcpt_handle h)
     cudaFree(h->dE);
     cudaFree(h->dH);
     cudaFree(h->dVT);
+    cudaFree(h->dFc);
     cudaFree(h->dCoup);
     cudaFree(h->dR);
     cudaFree(h->dS1);

@@ -68,8 +68,15 @@ cudaError_t launch_half_fp64(const DimerDesc* d_desc, int nd, int max_rows, int 
                              const double* Cpool, double* H, cudaStream_t s);
 
 // FP32 first half with compensated (TwoProduct/TwoSum) accumulation.
+// scratch: kFp32cCounterBytes, then `slots` slots (one per resident CTA) of
+// slot_bytes >= fp32c_slot_bytes of every dimer; slots = 0 runs the kernel
+// that needs no scratch.
+constexpr size_t kFp32cCounterBytes = 256;
+constexpr int kFp32cSlotsPerSM = 2;
+size_t fp32c_slot_bytes(int nX, int oY);
 cudaError_t launch_half_fp32c(const DimerDesc* d_desc, int nd, int max_rows, int max_occ,
-                              const float* Cf, float* H, cudaStream_t s);
+                              const float* Cf, float* H, void* scratch, int slots, size_t slot_bytes,
+                              cudaStream_t s);
 
 // Second half of monomers above 32 AO: one CTA per task = a range of one
 // dimer's occupied pairs; the tasks of a dimer are consecutive.
