@@ -146,7 +146,7 @@ struct mcpt_ctx {
         size_t fin_off;              // byte offset of the wave's tasks in dFin
         int ntasks;                  // 0: one CTA per dimer (<= 32 AO)
         size_t part_off;             // first partial (pairs of doubles) in dPart
-        int fin_warps;               // warps per CTA of the 32-AO second half
+        FinSplit fin;                // the 32-AO second half's split
     };
     // A plan is the host work of a run that does not change between runs of
     // the same dimer range and precision (descriptors, waves, tensor maps and
@@ -1047,7 +1047,9 @@ static mcpt_status build_plan(mcpt_handle h, mcpt_ctx::Plan& P, int first, int c
 
     mcpt_status st = upload_static(h);
     if (st) return st;
-    if ((st = ensure(h, &P.dDesc, &P.capDesc, ndesc * sizeof(DimerDesc)))) return st;
+    // the descriptors, then the second half's arrival counters (one each)
+    if ((st = ensure(h, &P.dDesc, &P.capDesc, ndesc * (sizeof(DimerDesc) + sizeof(unsigned))))) return st;
+    unsigned* const fin_cnt = reinterpret_cast<unsigned*>(P.dDesc + ndesc);
     if ((st = ensure_shared(h, &h->dH, &h->capH, max_wave_h))) return st;
     if (P.fc_slots &&
         ensure_shared(h, &h->dFc, &h->capFc, kFp32cCounterBytes + P.fc_slots * P.fc_slot_bytes) != MCPT_OK) {
@@ -1173,6 +1175,7 @@ static mcpt_status build_plan(mcpt_handle h, mcpt_ctx::Plan& P, int first, int c
         CK(h, cudaStreamSynchronize(h->stream));   // tab is pageable and goes out of scope
     }
     CK(h, cudaMemcpyAsync(P.dDesc, P.hDesc.data(), ndesc * sizeof(DimerDesc), cudaMemcpyHostToDevice, h->stream));
+    CK(h, cudaMemsetAsync(fin_cnt, 0, ndesc * sizeof(unsigned), h->stream));
     if (!fold.empty())
         CK(h, cudaMemcpyAsync(P.dFold, fold.data(), fold.size() * sizeof(int), cudaMemcpyHostToDevice, h->stream));
     P.nfold = (int)fold.size() / 3;
@@ -1222,13 +1225,14 @@ static mcpt_status build_plan(mcpt_handle h, mcpt_ctx::Plan& P, int first, int c
             wv.max_occ = std::max(wv.max_occ, std::max(dd.oX, dd.oY));
             wv.max_ao = std::max(wv.max_ao, std::max(dd.nX, dd.nY));
         }
-        wv.fin_warps = 4;
+        wv.fin = FinSplit{4, 1, nullptr};
         if (wv.max_ao <= 32) {
             const int form = prec == MCPT_FP64E ? FIN_FF
                              : fp64_data(prec)  ? FIN_F64
                              : h->fp64_epilogue ? FIN_F32_F64EPI
                                                 : FIN_F32_PAIRS;
-            wv.fin_warps = finish_w32_warps(P.hDesc.data() + wv.b, wv.nd, form);
+            wv.fin = finish_w32_split(P.hDesc.data() + wv.b, wv.nd, form, h->sms);
+            wv.fin.cnt = fin_cnt + wv.b;
         }
         if (is_tensor_form(prec)) {
             char tcerr[256] = {0};
@@ -1315,15 +1319,15 @@ static mcpt_status enqueue_run(mcpt_handle h, const mcpt_ctx::Plan& P, const std
         double* part = wv.ntasks ? P.dPart + 2 * wv.part_off : nullptr;
         if (prec == MCPT_FP64E && wv.max_ao <= 32)   // H as FP32 pairs (the tensor-core launch's h_pairs)
             CK(h, launch_finish_ff(wd, wv.nd, wv.max_ao, h->dC, h->dE, h->dH, h->dE2,
-                                   P.coupling ? static_cast<double*>(h->dVT) : nullptr, wv.fin_warps, h->stream));
+                                   P.coupling ? static_cast<double*>(h->dVT) : nullptr, wv.fin, h->stream));
         else if (fp64_data(prec))
-            CK(h, launch_finish_fp64(wd, wv.nd, wv.max_ao, h->dC, h->dE, static_cast<const double*>(h->dH), h->dE2,
+            CK(h, launch_finish_fp64(wd, wv.nd, wv.max_ao, h->dC, h->dE, static_cast<double*>(h->dH), h->dE2,
                                      tasks, wv.ntasks, part, P.coupling ? static_cast<double*>(h->dVT) : nullptr,
-                                     wv.fin_warps, h->stream));
+                                     wv.fin, h->stream));
         else
-            CK(h, launch_finish_fp32(wd, wv.nd, wv.max_ao, h->dCf, h->dE, static_cast<const float*>(h->dH), h->dE2,
+            CK(h, launch_finish_fp32(wd, wv.nd, wv.max_ao, h->dCf, h->dE, static_cast<float*>(h->dH), h->dE2,
                                      tasks, wv.ntasks, part, P.coupling ? static_cast<float*>(h->dVT) : nullptr,
-                                     h->fp64_epilogue, wv.fin_warps, h->stream));
+                                     h->fp64_epilogue, wv.fin, h->stream));
         launches += wv.ntasks ? 2 : 1;
         if (ev) CK(h, cudaEventRecord((*ev)[2 + 2 * w], h->stream));
     }

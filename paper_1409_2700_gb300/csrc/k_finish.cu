@@ -19,7 +19,8 @@
 // products with D and the sums over b, added to the FP64 sums once per pair --
 // no FP64 operation per term.  The FP64-pipe variant of that epilogue (five
 // FP64 operations per term) stays selectable for comparison.
-// Monomers of at most 32 AO: one CTA per dimer, one warp per occupied pair.
+// Monomers of at most 32 AO: one warp per occupied pair, a dimer's pairs over
+// one or more CTAs.
 // Larger ones: register-tiled GEMMs, one CTA per range of a dimer's pairs,
 // the ranges' partial sums added per dimer in range order.  Every sum has a
 // fixed order: the energies are deterministic run to run, with no atomics.
@@ -94,10 +95,7 @@ __device__ __forceinline__ void energy_terms(T v, T vk, double x, double& ej, do
 // one step ahead: H1 of this pair streams in during the H0 work, H0 of the
 // next pair during the H1 work, so the warp rarely waits on memory.  VA
 // takes the place of H0 in its buffer.  Per-lane sums reduce in a fixed order.
-// W warps per CTA (4 or 5, chosen per wave by finish_w32_warps from the
-// occupancy of each and the rounds of one pair per warp a dimer takes: o_X o_Y
-// = 25 pairs fill five warps evenly, but at 166 registers five warps fit two
-// CTAs per SM against four warps' three, and four measured faster).
+// A dimer's pairs are dealt to `parts` CTAs of W warps (finish_w32_split).
 constexpr int kW32Slab = 32 * 33;      // one padded 32 x 32 tile (row stride 33)
 constexpr int kCS = 36;                // row stride of the staged C columns: 16-byte rows for vector
                                        // loads, lane rows 4 banks apart (4-way instead of 32-way)
@@ -194,6 +192,90 @@ __device__ __forceinline__ void slice_wait()
     __syncwarp();
 }
 
+// A warp's lanes' E_J and E_K sums by a fixed tree: the halves swap a sum
+// first, so that lanes 0-15 reduce E_J while 16-31 reduce E_K (five FP64
+// additions, not ten).  Lane 0 returns E_J, lane 16 E_K.
+__device__ __forceinline__ double pair_tree(double ej, double ek, int lane)
+{
+    const bool hi = lane >= 16;
+    double s = (hi ? ek : ej) + __shfl_xor_sync(0xffffffffu, hi ? ej : ek, 16);
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    return s;
+}
+
+// Where the sums of a dimer's pairs meet.  A CTA that has the whole dimer
+// keeps them in shared memory (up to kPairSums pairs).  Otherwise each pair's
+// two sums go into the first 16 bytes of the pair's own H_0 slice, which its
+// warp has read and nobody reads again (a slice has at least 2 x 2 elements;
+// written as words: slices of odd sizes are 4-byte aligned).
+constexpr int kPairSums = 64;
+
+__device__ __forceinline__ void put_pair_sums(double (*ps)[2], void* slice, int pr, bool local, double ej, double ek,
+                                              int lane)
+{
+    const double s = pair_tree(ej, ek, lane);
+    if ((lane & 15) != 0) return;
+    if (local) {
+        ps[pr][lane >> 4] = s;
+    } else {
+        unsigned* w = static_cast<unsigned*>(slice) + (lane >> 3);
+        const unsigned long long a = (unsigned long long)__double_as_longlong(s);
+        __stcg(w, (unsigned)a);
+        __stcg(w + 1, (unsigned)(a >> 32));
+    }
+}
+
+__device__ __forceinline__ void get_pair_sums(const void* slice, double& ej, double& ek)
+{
+    const unsigned* w = static_cast<const unsigned*>(slice);
+    const unsigned long long a = ((unsigned long long)__ldcg(w + 1) << 32) | __ldcg(w);
+    const unsigned long long b = ((unsigned long long)__ldcg(w + 3) << 32) | __ldcg(w + 2);
+    ej = __longlong_as_double((long long)a);
+    ek = __longlong_as_double((long long)b);
+}
+
+// End of one of a dimer's `parts` CTAs: the last to arrive (any of them: the
+// result does not depend on which) adds the dimer's pair sums -- lane l pairs
+// l, l + 32, ... in order, then the fixed tree -- so the energies are the same
+// bits however the pairs were dealt to warps and CTAs.  slices: the dimer's
+// first H_0 slice; stride: bytes from one to the next.  cnt: the dimer's
+// arrival counter, zero before the launch and again after it.
+__device__ __forceinline__ void finish_dimer(const double (*ps)[2], const char* slices, size_t stride, int pairs,
+                                             bool local, int parts, unsigned* cnt, double* E2)
+{
+    __shared__ int last;
+    if (parts > 1) {
+        __threadfence();
+        __syncthreads();
+        if (threadIdx.x == 0) last = atomicAdd(cnt, 1u) == (unsigned)parts - 1;
+        __syncthreads();
+        if (!last) return;
+        __threadfence();
+    } else {
+        __syncthreads();
+    }
+    if (threadIdx.x >= 32) return;
+    double ej = 0.0, ek = 0.0;
+    for (int p = threadIdx.x; p < pairs; p += 32) {
+        double a, b;
+        if (local) {
+            a = ps[p][0];
+            b = ps[p][1];
+        } else {
+            get_pair_sums(slices + p * stride, a, b);
+        }
+        ej += a;
+        ek += b;
+    }
+    const double s = pair_tree(ej, ek, threadIdx.x);
+    if (threadIdx.x == 0) {
+        E2[0] = 4.0 * s;
+        if (parts > 1) *cnt = 0;
+    }
+    if (threadIdx.x == 16) E2[1] = -2.0 * s;
+}
+
 // STORE: also write the dimer's (ia|jb) and T for the coupling (a separate
 // instantiation keeps the plain path's registers).  PAIRS (mixed forms only):
 // the energy terms on FP32 pairs, summed per (pair, a) and added to the FP64
@@ -201,17 +283,21 @@ __device__ __forceinline__ void slice_wait()
 template <typename T, bool STORE, bool PAIRS, int W>
 __global__ void __launch_bounds__(W * 32, W == 4 ? 3 : 2)
 k_finish_w32(const DimerDesc* __restrict__ dd, const T* __restrict__ C, const double* __restrict__ Epool,
-             const T* __restrict__ H, double* __restrict__ E2, T* __restrict__ VT)
+             T* H, double* __restrict__ E2, T* __restrict__ VT, int parts, unsigned* __restrict__ cnt)
 {
-    const DimerDesc& d = dd[blockIdx.x];
+    const int dimer = blockIdx.y, cta = blockIdx.x;
+    const DimerDesc& d = dd[dimer];
     const int nX = d.nX, nY = d.nY, oX = d.oX, oY = d.oY;
     const int vX = d.vX, vY = d.vY;
     const int rows = nX * nY, pairs = oX * oY;
+    const int pr0 = cta * pairs / parts, pr1 = (cta + 1) * pairs / parts;   // this CTA's pairs
+    __shared__ double ps[kPairSums][2];
+    const bool local = parts == 1 && pairs <= kPairSums;
     const T* CXv = C + d.cXv;                 // virtual columns
     const T* CYv = C + d.cYv;
     const double* eX = Epool + d.eX;          // occupied energies of this block
     const double* eY = Epool + d.eY;
-    const T* H0 = H + d.h_off;
+    T* H0 = H + d.h_off;
     const T* H1 = H + d.h_off + (long long)pairs * rows;
 
     extern __shared__ __align__(16) unsigned char smraw[];
@@ -225,9 +311,9 @@ k_finish_w32(const DimerDesc* __restrict__ dd, const T* __restrict__ C, const do
     [[maybe_unused]] T* const SV = buf + 2 * kW32Slab;        // FP32: (ib|ja) as [b][a] (stride 33)
 
     // the warp's first pair streams in while the block stages C and the energies
-    if (warp < pairs) {
-        prefetch_slice(buf, H0 + (long long)warp * rows, nX, nY, lane);
-        prefetch_slice(buf + kW32Slab, H1 + (long long)warp * rows, nY, nX, lane);
+    if (pr0 + warp < pr1) {
+        prefetch_slice(buf, H0 + (long long)(pr0 + warp) * rows, nX, nY, lane);
+        prefetch_slice(buf + kW32Slab, H1 + (long long)(pr0 + warp) * rows, nY, nX, lane);
     }
     {
         // all loads first (independent, in flight together), then the stores;
@@ -263,10 +349,10 @@ k_finish_w32(const DimerDesc* __restrict__ dd, const T* __restrict__ C, const do
     const bool store = STORE && d.vt_off >= 0;
     const long long mXc = (long long)d.oXt * vX, mYc = (long long)d.oYt * vY;
     T* const Vst = store ? VT + d.vt_off : nullptr;
-    double ej = 0.0, ek = 0.0;
     int x = 0;                                   // buffer holding this pair's H0
-    for (int pr = warp; pr < pairs; pr += W, x ^= 1) {
+    for (int pr = pr0 + warp; pr < pr1; pr += W, x ^= 1) {
         const int i = pr / oY, j = pr % oY;
+        double ej = 0.0, ek = 0.0;               // this pair's sums
         const double eija = (eX[i] + eY[j]) - ea;  // e_i + e_j - e_a of this lane
         [[maybe_unused]] const FF eijas = PAIRS ? ff_split(eija) : FF{0.f, 0.f};
         [[maybe_unused]] FF sj{0.f, 0.f}, sk{0.f, 0.f};   // this pair's sums over even b (PAIRS)
@@ -326,7 +412,7 @@ k_finish_w32(const DimerDesc* __restrict__ dd, const T* __restrict__ C, const do
                 for (int lam = 0; lam < 32; lam++) tk[lam] = dot32(SY + lam * 32, cx);
             }
             __syncwarp();                        // H1 consumed: the next pair's H0 streams into SY
-            if (nx < pairs) prefetch_slice(SY, H0 + (long long)nx * rows, nX, nY, lane);
+            if (nx < pr1) prefetch_slice(SY, H0 + (long long)nx * rows, nX, nY, lane);
             // ---- FP32: (ib|ja) of every b into this lane's column of SV, four
             // independent multiply-add chains at a time (each lane reads back
             // only its own column)
@@ -384,25 +470,15 @@ k_finish_w32(const DimerDesc* __restrict__ dd, const T* __restrict__ C, const do
             }
         }
         if constexpr (PAIRS) {
-            ej += ff_f64(sj);
-            ek += ff_f64(sk);
-            ej += ff_f64(sj1);
-            ek += ff_f64(sk1);
+            ej = ff_f64(sj) + ff_f64(sj1);
+            ek = ff_f64(sk) + ff_f64(sk1);
         }
         __syncwarp();                            // VA consumed: the next pair's H1 streams into SX
-        if (nx < pairs) prefetch_slice(SX, H1 + (long long)nx * rows, nY, nX, lane);
+        if (nx < pr1) prefetch_slice(SX, H1 + (long long)nx * rows, nY, nX, lane);
+        put_pair_sums(ps, H0 + (long long)pr * rows, pr, local, ej, ek, lane);
     }
-    __shared__ double red[2][W];
-    ej = warp_sum(ej);
-    ek = warp_sum(ek);
-    if (lane == 0) { red[0][warp] = ej; red[1][warp] = ek; }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double sj = 0.0, sk = 0.0;
-        for (int w = 0; w < W; w++) { sj += red[0][w]; sk += red[1][w]; }
-        E2[2 * d.slot + 0] = 4.0 * sj;
-        E2[2 * d.slot + 1] = -2.0 * sk;
-    }
+    finish_dimer(ps, reinterpret_cast<const char*>(H0), (size_t)rows * sizeof(T), pairs, local, parts, cnt + dimer,
+                 E2 + 2 * d.slot);
 }
 
 // ---------------------------------------------------------------------------
@@ -425,17 +501,21 @@ size_t w32_ff_smem_bytes(int W) { return (32 + 2 * (size_t)kFFSlab + 2 * (size_t
 template <bool STORE, int W>
 __global__ void __launch_bounds__(W * 32, 2)
 k_finish_w32_ff(const DimerDesc* __restrict__ dd, const double* __restrict__ C, const double* __restrict__ Epool,
-                const FF* __restrict__ H, double* __restrict__ E2, double* __restrict__ VT)
+                FF* H, double* __restrict__ E2, double* __restrict__ VT, int parts, unsigned* __restrict__ cnt)
 {
-    const DimerDesc& d = dd[blockIdx.x];
+    const int dimer = blockIdx.y, cta = blockIdx.x;
+    const DimerDesc& d = dd[dimer];
     const int nX = d.nX, nY = d.nY, oX = d.oX, oY = d.oY;
     const int vX = d.vX, vY = d.vY;
     const int rows = nX * nY, pairs = oX * oY;
+    const int pr0 = cta * pairs / parts, pr1 = (cta + 1) * pairs / parts;   // this CTA's pairs
+    __shared__ double ps[kPairSums][2];
+    const bool local = parts == 1 && pairs <= kPairSums;
     const double* CXv = C + d.cXv;            // virtual columns
     const double* CYv = C + d.cYv;
     const double* eX = Epool + d.eX;          // occupied energies of this block
     const double* eY = Epool + d.eY;
-    const FF* H0 = H + d.h_off;
+    FF* H0 = H + d.h_off;
     const FF* H1 = H + d.h_off + (long long)pairs * rows;
 
     extern __shared__ __align__(16) unsigned char smraw[];
@@ -445,9 +525,9 @@ k_finish_w32_ff(const DimerDesc* __restrict__ dd, const double* __restrict__ C, 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     FF* const buf = CYT + kFFSlab + warp * (2 * kFFSlab);   // two slice buffers
 
-    if (warp < pairs) {
-        prefetch_slice(buf, H0 + (long long)warp * rows, nX, nY, lane);
-        prefetch_slice(buf + kFFSlab, H1 + (long long)warp * rows, nY, nX, lane);
+    if (pr0 + warp < pr1) {
+        prefetch_slice(buf, H0 + (long long)(pr0 + warp) * rows, nX, nY, lane);
+        prefetch_slice(buf + kFFSlab, H1 + (long long)(pr0 + warp) * rows, nY, nX, lane);
     }
     for (int k = threadIdx.x; k < 32 * 32; k += W * 32) {
         const int m = k >> 5, a = k & 31;       // lanes along the contiguous index a
@@ -462,9 +542,8 @@ k_finish_w32_ff(const DimerDesc* __restrict__ dd, const double* __restrict__ C, 
     const bool store = STORE && d.vt_off >= 0;
     const long long mXc = (long long)d.oXt * vX, mYc = (long long)d.oYt * vY;
     double* const Vst = store ? VT + d.vt_off : nullptr;
-    double ej = 0.0, ek = 0.0;
     int x = 0;                                   // buffer holding this pair's H0
-    for (int pr = warp; pr < pairs; pr += W, x ^= 1) {
+    for (int pr = pr0 + warp; pr < pr1; pr += W, x ^= 1) {
         const int i = pr / oY, j = pr % oY;
         const FF eija = ff_split((eX[i] + eY[j]) - ea);   // e_i + e_j - e_a of this lane
         FF sj{0.f, 0.f}, sk{0.f, 0.f};
@@ -524,7 +603,7 @@ k_finish_w32_ff(const DimerDesc* __restrict__ dd, const double* __restrict__ C, 
                 for (int q = 0; q < kFFChains; q++) tk[lam + q] = acc[q];
             }
             __syncwarp();                        // H1 consumed: the next pair's H0 streams into SY
-            if (nx < pairs) prefetch_slice(SY, H0 + (long long)nx * rows, nX, nY, lane);
+            if (nx < pr1) prefetch_slice(SY, H0 + (long long)nx * rows, nX, nY, lane);
             // ---- denominators and energy sums, lane a over b
 #pragma unroll 1
             for (int b = 0; b < vY; b++) {
@@ -548,22 +627,12 @@ k_finish_w32_ff(const DimerDesc* __restrict__ dd, const double* __restrict__ C, 
                 }
             }
         }
-        ej += ff_f64(sj);
-        ek += ff_f64(sk);
         __syncwarp();                            // VA consumed: the next pair's H1 streams into SX
-        if (nx < pairs) prefetch_slice(SX, H1 + (long long)nx * rows, nY, nX, lane);
+        if (nx < pr1) prefetch_slice(SX, H1 + (long long)nx * rows, nY, nX, lane);
+        put_pair_sums(ps, H0 + (long long)pr * rows, pr, local, ff_f64(sj), ff_f64(sk), lane);
     }
-    __shared__ double red[2][W];
-    ej = warp_sum(ej);
-    ek = warp_sum(ek);
-    if (lane == 0) { red[0][warp] = ej; red[1][warp] = ek; }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double sjt = 0.0, skt = 0.0;
-        for (int w = 0; w < W; w++) { sjt += red[0][w]; skt += red[1][w]; }
-        E2[2 * d.slot + 0] = 4.0 * sjt;
-        E2[2 * d.slot + 1] = -2.0 * skt;
-    }
+    finish_dimer(ps, reinterpret_cast<const char*>(H0), (size_t)rows * sizeof(FF), pairs, local, parts, cnt + dimer,
+                 E2 + 2 * d.slot);
 }
 
 // ---------------------------------------------------------------------------
@@ -804,8 +873,8 @@ __global__ void k_finish_sum(const DimerDesc* __restrict__ dd, int nd, const Fin
 }
 
 template <typename T, bool PAIRS, int W>
-cudaError_t launch_w32(const DimerDesc* d_desc, int nd, const T* C, const double* Epool, const T* H, double* E2,
-                       T* VT, cudaStream_t s)
+cudaError_t launch_w32(const DimerDesc* d_desc, int nd, const T* C, const double* Epool, T* H, double* E2,
+                       T* VT, FinSplit sp, cudaStream_t s)
 {
     const size_t smem = w32_smem_bytes<T>(W);
     auto fn = VT ? k_finish_w32<T, true, PAIRS, W> : k_finish_w32<T, false, PAIRS, W>;
@@ -815,19 +884,19 @@ cudaError_t launch_w32(const DimerDesc* d_desc, int nd, const T* C, const double
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
     if (e != cudaSuccess) return e;
-    fn<<<nd, W * 32, smem, s>>>(d_desc, C, Epool, H, E2, VT);
+    fn<<<dim3(sp.parts, nd), W * 32, smem, s>>>(d_desc, C, Epool, H, E2, VT, sp.parts, sp.cnt);
     return cudaGetLastError();
 }
 
 template <typename T, bool PAIRS>
 cudaError_t launch_finish(const DimerDesc* d_desc, int nd, int max_ao, const T* C, const double* Epool,
-                          const T* H, double* E2, const FinTask* tasks, int ntasks, double* part, T* VT,
-                          int w32_warps, cudaStream_t s)
+                          T* H, double* E2, const FinTask* tasks, int ntasks, double* part, T* VT,
+                          FinSplit sp, cudaStream_t s)
 {
     if (nd <= 0) return cudaSuccess;
     if (max_ao <= 32)
-        return w32_warps == 5 ? launch_w32<T, PAIRS, 5>(d_desc, nd, C, Epool, H, E2, VT, s)
-                              : launch_w32<T, PAIRS, 4>(d_desc, nd, C, Epool, H, E2, VT, s);
+        return sp.warps == 5 ? launch_w32<T, PAIRS, 5>(d_desc, nd, C, Epool, H, E2, VT, sp, s)
+                             : launch_w32<T, PAIRS, 4>(d_desc, nd, C, Epool, H, E2, VT, sp, s);
     if (!tasks || ntasks <= 0 || !part) return cudaErrorInvalidValue;
     const size_t smem = tiled_smem_bytes<T>(max_ao);
     if (smem > 227 * 1024) return cudaErrorInvalidValue;
@@ -843,41 +912,16 @@ cudaError_t launch_finish(const DimerDesc* d_desc, int nd, int max_ao, const T* 
 }
 
 template <int W>
-cudaError_t launch_finish_ff_t(const DimerDesc* d_desc, int nd, const double* C, const double* Epool, const FF* H,
-                               double* E2, double* VT, cudaStream_t s)
+cudaError_t launch_finish_ff_t(const DimerDesc* d_desc, int nd, const double* C, const double* Epool, FF* H,
+                               double* E2, double* VT, FinSplit sp, cudaStream_t s)
 {
     if (nd <= 0) return cudaSuccess;
     const size_t smem = w32_ff_smem_bytes(W);
     auto fn = VT ? k_finish_w32_ff<true, W> : k_finish_w32_ff<false, W>;
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    fn<<<nd, W * 32, smem, s>>>(d_desc, C, Epool, H, E2, VT);
+    fn<<<dim3(sp.parts, nd), W * 32, smem, s>>>(d_desc, C, Epool, H, E2, VT, sp.parts, sp.cnt);
     return cudaGetLastError();
-}
-
-// CTAs of the 32-AO second half resident per SM with W warps (the plain
-// instantiation of the form; 0 if the query fails).
-template <int W>
-int w32_ctas_per_sm(int form)
-{
-    int n = 0, dev = 0, max_smem = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    cudaError_t e = cudaErrorInvalidValue;
-    auto occ = [&](auto fn, size_t smem) {
-        if ((int)smem > max_smem) return cudaErrorInvalidValue;
-        cudaError_t r = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (r == cudaSuccess && form != FIN_FF)
-            r = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-        return r != cudaSuccess ? r : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, W * 32, smem);
-    };
-    switch (form) {
-    case FIN_F64: e = occ(k_finish_w32<double, false, false, W>, w32_smem_bytes<double>(W)); break;
-    case FIN_F32_PAIRS: e = occ(k_finish_w32<float, false, true, W>, w32_smem_bytes<float>(W)); break;
-    case FIN_F32_F64EPI: e = occ(k_finish_w32<float, false, false, W>, w32_smem_bytes<float>(W)); break;
-    case FIN_FF: e = occ(k_finish_w32_ff<false, W>, w32_ff_smem_bytes(W)); break;
-    }
-    return e == cudaSuccess ? n : 0;
 }
 
 // Split dimers: the blocks' terms added in block order.
@@ -1034,46 +1078,50 @@ __global__ void k_check_finite4(const double* __restrict__ x, int d0, int d1, in
 }  // namespace
 
 cudaError_t launch_finish_fp64(const DimerDesc* d_desc, int nd, int max_ao, const double* Cpool,
-                               const double* Epool, const double* H, double* E2, const FinTask* tasks,
-                               int ntasks, double* part, double* VT, int w32_warps, cudaStream_t s)
+                               const double* Epool, double* H, double* E2, const FinTask* tasks,
+                               int ntasks, double* part, double* VT, FinSplit sp, cudaStream_t s)
 {
-    return launch_finish<double, false>(d_desc, nd, max_ao, Cpool, Epool, H, E2, tasks, ntasks, part, VT,
-                                        w32_warps, s);
+    return launch_finish<double, false>(d_desc, nd, max_ao, Cpool, Epool, H, E2, tasks, ntasks, part, VT, sp, s);
 }
 
 cudaError_t launch_finish_fp32(const DimerDesc* d_desc, int nd, int max_ao, const float* Cf,
-                               const double* Epool, const float* H, double* E2, const FinTask* tasks,
-                               int ntasks, double* part, float* VT, bool fp64_epilogue, int w32_warps,
+                               const double* Epool, float* H, double* E2, const FinTask* tasks,
+                               int ntasks, double* part, float* VT, bool fp64_epilogue, FinSplit sp,
                                cudaStream_t s)
 {
     return fp64_epilogue
-               ? launch_finish<float, false>(d_desc, nd, max_ao, Cf, Epool, H, E2, tasks, ntasks, part, VT,
-                                             w32_warps, s)
-               : launch_finish<float, true>(d_desc, nd, max_ao, Cf, Epool, H, E2, tasks, ntasks, part, VT,
-                                            w32_warps, s);
+               ? launch_finish<float, false>(d_desc, nd, max_ao, Cf, Epool, H, E2, tasks, ntasks, part, VT, sp, s)
+               : launch_finish<float, true>(d_desc, nd, max_ao, Cf, Epool, H, E2, tasks, ntasks, part, VT, sp, s);
 }
 
 cudaError_t launch_finish_ff(const DimerDesc* d_desc, int nd, int max_ao, const double* Cpool, const double* Epool,
-                             const void* H, double* E2, double* VT, int w32_warps, cudaStream_t s)
+                             void* H, double* E2, double* VT, FinSplit sp, cudaStream_t s)
 {
     if (max_ao > 32) return cudaErrorInvalidValue;
-    const FF* Hf = static_cast<const FF*>(H);
-    return w32_warps == 5 ? launch_finish_ff_t<5>(d_desc, nd, Cpool, Epool, Hf, E2, VT, s)
-                          : launch_finish_ff_t<4>(d_desc, nd, Cpool, Epool, Hf, E2, VT, s);
+    FF* Hf = static_cast<FF*>(H);
+    return sp.warps == 5 ? launch_finish_ff_t<5>(d_desc, nd, Cpool, Epool, Hf, E2, VT, sp, s)
+                         : launch_finish_ff_t<4>(d_desc, nd, Cpool, Epool, Hf, E2, VT, sp, s);
 }
 
-int finish_w32_warps(const DimerDesc* h, int nd, int form)
+// One round (a warp per pair) per CTA of four warps: the CTAs of a dimer run
+// on different SMs, so a wave of few dimers fills the chip instead of one SM
+// per dimer, and the CTAs' fine grain evens out the end of a larger wave.
+// Measured in us, one CTA of four warps per dimer against this: FP32, 1 / 28 /
+// 158 / 227 dimers 62 / 62 / 84 / 87 -> 17 / 22 / 54 / 70; FP64 (31 us of FP64
+// pipe per pair) 1 / 158 / 1036 dimers 1026 / 1682 / 5965 -> 154 / 952 / 5574;
+// FP64E 364 / 531 / 2117 -> 66 / 346 / 2065.  Five warps where they keep a
+// wave at one CTA per SM and four do not (28 dimers of 25 pairs: FP64 265 ->
+// 176).  FP32 waves of more than six dimers per SM are bound by the FP32
+// pipes either way, and staging the coefficients once per dimer is then the
+// cheaper: 1036 dimers 256 against 266, 2248 dimers 513 against 557.
+FinSplit finish_w32_split(const DimerDesc* h, int nd, int form, int sms)
 {
-    // a dimer's CTA takes ceil(pairs / W) rounds of one pair per warp; the
-    // wave's time goes as the rounds over the CTAs an SM holds at once
-    double t[2] = {0.0, 0.0};
-    const int ctas[2] = {w32_ctas_per_sm<4>(form), w32_ctas_per_sm<5>(form)};
-    if (form == FIN_FF) return 4;   // five warps per CTA measured slower for the FP32-pair form
-    for (int w = 0; w < 2; w++) {
-        if (ctas[w] <= 0) return 4;
-        for (int k = 0; k < nd; k++) t[w] += (double)((h[k].oX * h[k].oY + 3 + w) / (4 + w)) / ctas[w];
-    }
-    return t[1] < t[0] ? 5 : 4;
+    int pairs = 1;
+    for (int k = 0; k < nd; k++) pairs = std::max(pairs, h[k].oX * h[k].oY);
+    if ((form == FIN_F32_PAIRS || form == FIN_F32_F64EPI) && nd > 6 * sms) return FinSplit{4, 1, nullptr};
+    const int p4 = (pairs + 3) / 4, p5 = (pairs + 4) / 5;
+    const bool five = (long long)nd * p5 <= sms && (long long)nd * p4 > sms;
+    return five ? FinSplit{5, p5, nullptr} : FinSplit{4, p4, nullptr};
 }
 
 void finish_tasks(const DimerDesc* h, int nd, int fma_per_task, std::vector<FinTask>* out)

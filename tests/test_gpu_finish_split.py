@@ -1,0 +1,52 @@
+"""The 32-AO second half deals a dimer's occupied pairs to one or several CTAs
+by the size of the wave; the energies do not depend on how (marked gpu).
+
+A chain of more dimers than the one-CTA rule's line (six per SM), run at once,
+against the same dimers run as short ranges, whose pairs are spread over CTAs:
+the same bits.  Sizes: odd slices (their pair sums are kept at 4-byte aligned
+places), one pair, and more pairs (81) than the CTA keeps in shared memory.
+The first dimers also against the oracle, at the forms' bounds for few-term
+dimers (test_gpu_parity)."""
+import numpy as np
+import pytest
+
+import oracle
+from helpers import rand_dimer
+
+pytestmark = pytest.mark.gpu
+
+M = pytest.importorskip("paper_1409_2700_gb300")
+
+SIZES = {"fp64": [(3, 1), (5, 2), (12, 9), (7, 3)], "fp32c": [(3, 1), (5, 2), (12, 9), (7, 3)],
+         "tf32": [(4, 1), (6, 2), (14, 9), (8, 3)], "fp64e": [(4, 1), (6, 2), (14, 5), (8, 3)]}
+TOL = {"fp64": 1e-12, "fp32c": 2e-6, "tf32": 2e-3, "fp64e": 5e-12}
+ND = 6 * 160 + 8
+
+
+@pytest.mark.parametrize("prec", list(SIZES))
+def test_energies_do_not_depend_on_the_split(prec):
+    sizes = SIZES[prec]
+    rng = np.random.default_rng(11)
+    kinds = [rand_dimer(rng, sizes[k][0], sizes[(k + 1) % 4][0], sizes[k][1], sizes[(k + 1) % 4][1]) for k in range(4)]
+    mono = [(kinds[k][2], kinds[k][3], sizes[k][1]) for k in range(4)]
+    with M.Context(precision=prec) as ctx:
+        for m in range(ND + 1):
+            ctx.add_monomer(*mono[m % 4])
+        for d in range(ND):
+            A, K = kinds[d % 4][:2]
+            s = 1.0 + d / ND
+            ctx.add_dimer(d, d + 1, np.concatenate([A.ravel() * s, K.ravel() * s]), M.MCPT_AO_BLOCKS)
+        ctx.run()
+        whole = ctx.energies()[2].copy()
+        ctx.run(0, 6)
+        ctx.run(6, 1)
+        ctx.run(7, 30)
+        parts = ctx.energies()[2]
+        assert np.array_equal(parts, whole)
+    for d in range(4):
+        A, K = kinds[d][:2]
+        CX, eX, oX = mono[d]
+        CY, eY, oY = mono[(d + 1) % 4]
+        s = 1.0 + d / ND
+        ref = oracle.dimer(A * s, K * s, CX, eX, CY, eY, oX, oY)
+        assert np.all(np.abs(whole[d] - ref) <= TOL[prec] * abs(ref[0])), (d, whole[d], ref)
