@@ -138,7 +138,7 @@ struct mcpt_ctx {
     size_t capLists = 0;
     bool lists_dirty = true;
     double* dTot = nullptr;
-    int* dFlag = nullptr;            // [0] validation flag, [1] device wait status
+    int* dFlag = nullptr;            // [0] validation flag, [1] device wait status, [2] the reduction's counter
 
     struct Wave {
         int b, nd, max_rows, max_occ, max_ao;
@@ -332,6 +332,9 @@ bool all_finite(const double* x, size_t n)
         if (!std::isfinite(x[k])) return false;
     return true;
 }
+
+// The reductions' arrival counter (zeroed at creation; each launch leaves it zero).
+unsigned* reduce_counter(mcpt_ctx* h) { return reinterpret_cast<unsigned*>(h->dFlag + 2); }
 
 bool is_tensor_form(mcpt_precision p)
 {
@@ -1336,7 +1339,7 @@ static mcpt_status enqueue_run(mcpt_handle h, const mcpt_ctx::Plan& P, const std
         launches++;
     }
     MonomerLists L{h->dLists, h->dLists + N + 1, N};
-    CK(h, launch_reduce(h->dE2, D, L, h->dMon, h->dTot, h->dTot + 2, h->stream));
+    CK(h, launch_reduce(h->dE2, D, L, h->dMon, h->dTot, h->dTot + 2, reduce_counter(h), h->stream));
     if (P.coupling) {
         const char* tab = static_cast<const char*>(h->dCoup);
         const CoupTile* tiles = reinterpret_cast<const CoupTile*>(tab + P.off_tiles);
@@ -1351,7 +1354,7 @@ static mcpt_status enqueue_run(mcpt_handle h, const mcpt_ctx::Plan& P, const std
                                        h->stream));
         launches += (P.ntile[0] > 0) + (P.ntile[1] > 0) + (P.ntile[2] > 0);
     }
-    launches += 2;   // the reduction: partial sums, then their merge
+    launches++;      // the reduction
     if (ev) CK(h, cudaEventRecord((*ev)[2 * W + 1], h->stream));
     *launches_out = launches;
     return MCPT_OK;
@@ -1665,7 +1668,7 @@ mcpt_status mcpt_run_df(mcpt_handle h)
                     base + tab, reinterpret_cast<double*>(base + tab + halfb), E2, h->stream));
     MonomerLists L{h->dDfLists, h->dDfLists + N + 1, N};
     CK(h, launch_reduce(E2, D, L, E2 + 2 * (size_t)D, E2 + 2 * (size_t)D + 2 * (size_t)N,
-                        E2 + 2 * (size_t)D + 2 * (size_t)N + 2, h->stream));
+                        E2 + 2 * (size_t)D + 2 * (size_t)N + 2, reduce_counter(h), h->stream));
     CK(h, cudaStreamSynchronize(h->stream));   // the host tables go out of scope
     h->df_ran = true;
     return MCPT_OK;

@@ -948,9 +948,6 @@ __device__ __forceinline__ void neumaier_add(double& s, double& c, double v)
     s = t;
 }
 
-constexpr int kRedThreads = 256;
-constexpr int kMonWarps = kRedThreads / 32;   // per-monomer sums: one warp per monomer
-
 // Knuth's TwoSum of two compensated sums (s, c) and (s2, c2) into (s, c).
 __device__ __forceinline__ void twosum_pair(double& s, double& c, double s2, double c2)
 {
@@ -961,92 +958,83 @@ __device__ __forceinline__ void twosum_pair(double& s, double& c, double s2, dou
     s = t;
 }
 
-// Blocks [0, nbm): one warp per monomer.  Lane l sums half of the terms of
-// the monomer's dimers l, l + 32, ... of its list (Neumaier), and a fixed
-// shuffle tree merges the 32 lane sums (TwoSum per merge): the list's loads
-// are in flight together instead of one dependent load pair per dimer.
-// Blocks [nbm, nbm + nbt): lattice-total partials, block b over a fixed
-// contiguous range of the dimer list, its threads over fixed sub-chunks
-// (Neumaier), merged by a fixed pairwise tree (TwoSum keeps each merge's
-// rounding); k_total_merge then adds the block partials by the same tree.
-// Long dependent FP64 chains are slow on GB300 and one SM's FP64 pipe is
-// small, so the work is spread over many blocks; the partition depends only
-// on the dimer and monomer counts, so every run gives the same bits.
-__device__ __forceinline__ void twosum_merge(double* part, int t, int w)
+// The 32 lanes' compensated sums of J and K, (sj, cj) and (sk, ck), merged by
+// a fixed tree of TwoSums: the halves of the warp swap a sum first, so that
+// lanes 0-15 merge J while lanes 16-31 merge K (one dependent TwoSum per level
+// instead of two).  Returns J's sum in lanes 0-15, K's in 16-31.
+__device__ __forceinline__ void warp_merge(double sj, double cj, double sk, double ck, int lane, double& s, double& c)
 {
+    const bool hi = lane >= 16;
+    s = hi ? sk : sj;
+    c = hi ? ck : cj;
+    const double s2 = __shfl_xor_sync(0xffffffffu, hi ? sj : sk, 16);
+    const double c2 = __shfl_xor_sync(0xffffffffu, hi ? cj : ck, 16);
+    twosum_pair(s, c, s2, c2);
 #pragma unroll
-    for (int f = 0; f < 4; f += 2) {
-        const double a = part[f * kRedThreads + t], b = part[f * kRedThreads + t + w];
-        const double s = a + b;
-        const double bp = s - a;
-        const double err = (a - (s - bp)) + (b - bp);
-        part[f * kRedThreads + t] = s;
-        part[(f + 1) * kRedThreads + t] = part[(f + 1) * kRedThreads + t] + part[(f + 1) * kRedThreads + t + w] + err;
+    for (int o = 8; o > 0; o >>= 1) {
+        const double s3 = __shfl_xor_sync(0xffffffffu, s, o), c3 = __shfl_xor_sync(0xffffffffu, c, o);
+        twosum_pair(s, c, s3, c3);
     }
 }
 
-__global__ void __launch_bounds__(kRedThreads)
-k_reduce(const double* __restrict__ E2, int nd, MonomerLists L, double* __restrict__ mon, int nbm, int nbt,
-         double* __restrict__ partials)
+// One warp per block.  Blocks [0, n_mon): a monomer each; lane l sums half of
+// the terms of the monomer's dimers l, l + 32, ... of its list (Neumaier), and
+// the warp tree merges the lanes: the list's loads are in flight together.
+// Blocks [n_mon, n_mon + nbt): the lattice total, block b over a fixed
+// contiguous range of the dimer list, its lanes over fixed strides (Neumaier),
+// merged by the warp tree; the last of several blocks to arrive merges the
+// block sums the same way (cnt: zero before the launch and again after it).
+// Bound by dependent FP64 additions and loads.  An SM's FP64 pipe takes 16
+// cycles for one warp's addition, so warps that share an SM wait on each
+// other: single-warp blocks spread them over the chip.  One launch instead of
+// two with shared-memory trees of both sums over 256 threads.  The partition
+// depends only on the dimer and monomer counts, so every run gives the same
+// bits.
+__global__ void __launch_bounds__(32)
+k_reduce(const double* __restrict__ E2, int nd, MonomerLists L, double* __restrict__ mon, int nbt,
+         double* __restrict__ partials, double* __restrict__ total, unsigned* __restrict__ cnt)
 {
-    if ((int)blockIdx.x < nbm) {
-        const int m = blockIdx.x * kMonWarps + (int)(threadIdx.x >> 5), lane = threadIdx.x & 31;
-        if (m >= L.n_mon) return;                 // whole warps
-        double sj = 0, cj = 0, sk = 0, ck = 0;
+    const int lane = threadIdx.x;
+    double sj = 0, cj = 0, sk = 0, ck = 0, s, c;
+    if ((int)blockIdx.x < L.n_mon) {
+        const int m = blockIdx.x;
         for (int k = L.start[m] + lane; k < L.start[m + 1]; k += 32) {
             const int dslot = L.list[k];
             neumaier_add(sj, cj, 0.5 * E2[2 * dslot]);
             neumaier_add(sk, ck, 0.5 * E2[2 * dslot + 1]);
         }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const double sj2 = __shfl_down_sync(0xffffffffu, sj, o), cj2 = __shfl_down_sync(0xffffffffu, cj, o);
-            const double sk2 = __shfl_down_sync(0xffffffffu, sk, o), ck2 = __shfl_down_sync(0xffffffffu, ck, o);
-            twosum_pair(sj, cj, sj2, cj2);
-            twosum_pair(sk, ck, sk2, ck2);
-        }
-        if (lane == 0) {
-            mon[m] = sj + cj;
-            mon[L.n_mon + m] = sk + ck;
-        }
+        warp_merge(sj, cj, sk, ck, lane, s, c);
+        if ((lane & 15) == 0) mon[(lane >> 4) * L.n_mon + m] = s + c;
         return;
     }
-    __shared__ double part[4 * kRedThreads];
-    const int b = blockIdx.x - nbm, t = threadIdx.x;
+    const int b = blockIdx.x - L.n_mon;
     const int per = (nd + nbt - 1) / nbt;
     const int b0 = b * per, b1 = min(nd, b0 + per);
-    const int chunk = (per + kRedThreads - 1) / kRedThreads;
-    const int lo = b0 + t * chunk, hi = min(b1, lo + chunk);
-    double sj = 0, cj = 0, sk = 0, ck = 0;
-    for (int k = lo; k < hi; k++) {
+    for (int k = b0 + lane; k < b1; k += 32) {
         neumaier_add(sj, cj, E2[2 * k]);
         neumaier_add(sk, ck, E2[2 * k + 1]);
     }
-    part[t] = sj; part[kRedThreads + t] = cj; part[2 * kRedThreads + t] = sk; part[3 * kRedThreads + t] = ck;
-    __syncthreads();
-    for (int w = kRedThreads / 2; w > 0; w >>= 1) {
-        if (t < w) twosum_merge(part, t, w);
-        __syncthreads();
+    warp_merge(sj, cj, sk, ck, lane, s, c);
+    if (nbt > 1) {
+        unsigned arrived = 0;
+        if ((lane & 15) == 0) {
+            __stcg(partials + 4 * b + (lane >> 3), s);
+            __stcg(partials + 4 * b + (lane >> 3) + 1, c);
+            __threadfence();
+        }
+        __syncwarp();
+        if (lane == 0) arrived = atomicAdd(cnt, 1u);
+        if (__shfl_sync(0xffffffffu, arrived, 0) != (unsigned)nbt - 1) return;
+        __threadfence();
+        sj = cj = sk = ck = 0;
+        for (int k = lane; k < nbt; k += 32) {
+            twosum_pair(sj, cj, __ldcg(partials + 4 * k), __ldcg(partials + 4 * k + 1));
+            twosum_pair(sk, ck, __ldcg(partials + 4 * k + 2), __ldcg(partials + 4 * k + 3));
+        }
+        warp_merge(sj, cj, sk, ck, lane, s, c);
+        if (lane == 0) *cnt = 0;
     }
-    if (t < 4) partials[4 * b + t] = part[t * kRedThreads];
-}
-
-__global__ void __launch_bounds__(kRedThreads)
-k_total_merge(const double* __restrict__ partials, int nbt, double* __restrict__ total)
-{
-    __shared__ double part[4 * kRedThreads];
-    const int t = threadIdx.x;
-#pragma unroll
-    for (int f = 0; f < 4; f++) part[f * kRedThreads + t] = t < nbt ? partials[4 * t + f] : 0.0;
-    __syncthreads();
-    for (int w = kRedThreads / 2; w > 0; w >>= 1) {
-        if (t < w) twosum_merge(part, t, w);
-        __syncthreads();
-    }
-    if (t == 0) {
-        total[0] = part[0] + part[kRedThreads];
-        total[1] = part[2 * kRedThreads] + part[3 * kRedThreads];
-    }
+    if ((lane & 15) == 0) total[lane >> 4] = s + c;
 }
 
 __global__ void k_check_finite(const double* __restrict__ x, long long n, int* flag)
@@ -1147,15 +1135,11 @@ cudaError_t launch_fold(const int* fold, int nfold, double* E2, cudaStream_t s)
 }
 
 cudaError_t launch_reduce(const double* E2, int nd, MonomerLists lists, double* mon, double* total,
-                          double* scratch, cudaStream_t s)
+                          double* scratch, unsigned* cnt, cudaStream_t s)
 {
-    const int nbm = (lists.n_mon + kMonWarps - 1) / kMonWarps;
-    // about 512 dimers per total block, at most kReduceBlocks blocks
-    const int nbt = std::max(1, std::min(kReduceBlocks, (nd + 511) / 512));
-    k_reduce<<<nbm + nbt, kRedThreads, 0, s>>>(E2, nd, lists, mon, nbm, nbt, scratch);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    k_total_merge<<<1, kRedThreads, 0, s>>>(scratch, nbt, total);
+    // two dimers per lane of a total block, at most kReduceBlocks blocks
+    const int nbt = std::max(1, std::min(kReduceBlocks, (nd + 63) / 64));
+    k_reduce<<<lists.n_mon + nbt, 32, 0, s>>>(E2, nd, lists, mon, nbt, scratch, total, cnt);
     return cudaGetLastError();
 }
 

@@ -6,7 +6,10 @@ against the same dimers run as short ranges, whose pairs are spread over CTAs:
 the same bits.  Sizes: odd slices (their pair sums are kept at 4-byte aligned
 places), one pair, and more pairs (81) than the CTA keeps in shared memory.
 The first dimers also against the oracle, at the forms' bounds for few-term
-dimers (test_gpu_parity)."""
+dimers (test_gpu_parity); the lattice total and the monomer sums against the
+exact sums of the dimers' terms."""
+import math
+
 import numpy as np
 import pytest
 
@@ -37,7 +40,16 @@ def test_energies_do_not_depend_on_the_split(prec):
             s = 1.0 + d / ND
             ctx.add_dimer(d, d + 1, np.concatenate([A.ravel() * s, K.ravel() * s]), M.MCPT_AO_BLOCKS)
         ctx.run()
-        whole = ctx.energies()[2].copy()
+        mj, mk, pd, tot = ctx.energies()
+        whole = pd.copy()
+        # the compensated sums, over many blocks of dimers: one FP64 rounding
+        # of the exact sum (2^-53) and of the lanes' error terms, within 2^-51
+        for f, mon in ((0, mj), (1, mk)):
+            assert abs(tot[f] - math.fsum(pd[:, f])) <= 2.0 ** -51 * np.abs(pd[:, f]).sum()
+            both = np.zeros(ND + 1)
+            both[:-1] += 0.5 * pd[:, f]
+            both[1:] += 0.5 * pd[:, f]
+            assert np.all(np.abs(mon - both) <= 2.0 ** -51 * np.abs(pd[:, f]).max())
         ctx.run(0, 6)
         ctx.run(6, 1)
         ctx.run(7, 30)
