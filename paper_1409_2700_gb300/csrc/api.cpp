@@ -1621,25 +1621,31 @@ mcpt_status mcpt_run_df(mcpt_handle h)
     const size_t es = fp64 ? sizeof(double) : sizeof(float);
     std::vector<DfDim> dims(D);
     long long hoff = 0;
-    int poff = 0, max_naux = 0, max_pairs = 0, max_on = 0, max_v = 0;
+    int poff = 0;
+    DfMax mx{};
     for (int d = 0; d < D; d++) {
         const DfRec& r = h->dfs[d];
         const MonomerRec& mX = h->mons[r.X];
         const MonomerRec& mY = h->mons[r.Y];
         const int nX = mX.nao, nY = mY.nao, oX = mX.nocc, oY = mY.nocc, vX = nX - oX, vY = nY - oY;
-        // shared memory of the half-transformation: B^Q, C_X, C_Y and the occupied rows
+        // shared memory of the FP64 half-transformation: B^Q, C_X, C_Y and the
+        // occupied rows; both forms keep its size limit
         const int on = (nX + nY) * (nX + nY) + nX * nX + nY * nY + (oX + oY) * (nX + nY);
         if ((size_t)on * es > (size_t)200 * 1024)
             return fail(h, MCPT_EUNSUPPORTED, "mcpt_run_df: dimer %d (%d + %d AO) needs %zu bytes of shared memory",
                         d, nX, nY, (size_t)on * es);
         dims[d] = DfDim{r.B, r.naux, nX, nY, oX, oY, mX.offC, mY.offC, mX.offE, mY.offE, r.s, hoff, poff, d};
-        hoff += (long long)r.naux * ((long long)oX * vX + (long long)oY * vY + (long long)oX * vY + (long long)oY * vX);
+        hoff += df_half_elems(fp64, r.naux, nX, nY, oX, oY);
         hoff = (hoff + 63) / 64 * 64;
         poff += oX * oY;
-        max_naux = std::max(max_naux, r.naux);
-        max_pairs = std::max(max_pairs, oX * oY);
-        max_on = std::max(max_on, on);
-        max_v = std::max(max_v, std::max(vX, vY));
+        mx.naux = std::max(mx.naux, r.naux);
+        mx.occ = std::max(mx.occ, std::max(oX, oY));
+        mx.v = std::max(mx.v, std::max(vX, vY));
+        int ue = 0, ce = 0;
+        df_smem_elems(nX, nY, oX, oY, &ue, &ce);
+        mx.u_elems = std::max(mx.u_elems, ue);
+        mx.c_elems = std::max(mx.c_elems, ce);
+        mx.b_elems = std::max(mx.b_elems, on);
     }
     // monomer lists of the density-fitted dimers (CSR, ascending dimer id)
     std::vector<int> cnt(N + 1, 0), lists(N + 1 + 2 * (size_t)D);
@@ -1664,8 +1670,8 @@ mcpt_status mcpt_run_df(mcpt_handle h)
     CK(h, cudaMemcpyAsync(base, dims.data(), (size_t)D * sizeof(DfDim), cudaMemcpyHostToDevice, h->stream));
     CK(h, cudaMemcpyAsync(h->dDfLists, lists.data(), lists.size() * sizeof(int), cudaMemcpyHostToDevice, h->stream));
     double* E2 = h->dDfOut;
-    CK(h, launch_df(fp64, reinterpret_cast<const DfDim*>(base), D, max_naux, max_pairs, max_on, max_v, h->dC, h->dE,
-                    base + tab, reinterpret_cast<double*>(base + tab + halfb), E2, h->stream));
+    CK(h, launch_df(fp64, reinterpret_cast<const DfDim*>(base), D, mx, h->dC, h->dE, base + tab,
+                    reinterpret_cast<double*>(base + tab + halfb), E2, h->sms, h->stream));
     MonomerLists L{h->dDfLists, h->dDfLists + N + 1, N};
     CK(h, launch_reduce(E2, D, L, E2 + 2 * (size_t)D, E2 + 2 * (size_t)D + 2 * (size_t)N,
                         E2 + 2 * (size_t)D + 2 * (size_t)N + 2, reduce_counter(h), h->stream));

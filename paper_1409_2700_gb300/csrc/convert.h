@@ -24,14 +24,15 @@ __device__ __forceinline__ unsigned tf32_from_f64_hi(unsigned hi)
     return e > 0 ? (sign | ((r - (896u << 10)) << 13)) : sign;
 }
 
-// FP32 from both words of a double, round half away from zero.
+// FP32 from both words of a double, round half away from zero.  The 32 bits
+// below the sign and the exponent's three high bits hold the exponent's low 8
+// bits, the 23 mantissa bits and the rounding bit; adding 1 rounds, and
+// flipping the top bit (subtracting 128 from the exponent modulo 256) rebiases
+// by 896, since 896 = 3 * 256 + 128: seven integer operations with the flush.
 __device__ __forceinline__ float f32_from_f64_bits(unsigned lo, unsigned hi)
 {
-    const unsigned sign = hi & 0x80000000u;
-    const int e = (int)((hi >> 20) & 0x7FFu) - 896;
-    unsigned m = ((unsigned)e << 23) | ((hi & 0xFFFFFu) << 3) | (lo >> 29);
-    m += (lo >> 28) & 1u;
-    return __uint_as_float(e > 0 ? (sign | m) : sign);
+    const unsigned v = (__funnelshift_l(lo, hi, 4) + 0x80000001u) >> 1;
+    return __uint_as_float((hi & 0x80000000u) | ((hi << 1) >= 0x70200000u ? v : 0u));   // 0x38100000 = 897 << 20
 }
 
 __device__ __forceinline__ float f32_from_f64(double x)

@@ -246,17 +246,26 @@ struct DfDim {
     int naux, nX, nY, oX, oY;
     int cX, cY, eX, eY;       // offsets of C and eps in the monomer pools
     double s;
-    long long h_off;          // half-transformed blocks: naux x (oX vX + oY vY + oX vY + oY vX) elements
-    int p_off;                // first pair partial (pairs of doubles)
+    long long h_off;          // half-transformed blocks (df_half_elems, a multiple of 4 elements from the start):
+                              //   xx [naux][oX][v_X], yy [naux][oY][v_Y], xy [naux][oX][v_Y], yx [naux][oY][v_X],
+                              //   FP32: rows padded with zeros to a multiple of 4 elements
+    int p_off;                // first partial (pairs of doubles; at most oX oY of a dimer are used)
     int id;                   // row of E2
 };
+// The largest of each over a launch's dimers.
+struct DfMax {
+    int naux, occ, v;                    // naux; max(oX, oY); max(vX, vY)
+    int u_elems, c_elems;                // FP32: shared elements of k_df_half (df_smem_elems)
+    int b_elems;                         // FP64: of k_df_half_fp64, n^2 + nX^2 + nY^2 + (oX + oY) n
+};
+// Occupied rows of one factor, and the columns of C, as k_df_half keeps them.
+void df_smem_elems(int nX, int nY, int oX, int oY, int* u_elems, int* c_elems);
+long long df_half_elems(bool fp64, int naux, int nX, int nY, int oX, int oY);
 // Terms of nd dimers into E2 (2 doubles each): FP64 arithmetic if fp64,
-// else FP32 (energy epilogue FP64).  max_on = max over dimers of the
-// half-transformation's shared elements n^2 + nX^2 + nY^2 + (oX + oY) n;
-// max_v = max(vX, vY); half: scratch of the half-transformed blocks;
-// part: 2 doubles per occupied pair.
-cudaError_t launch_df(bool fp64, const DfDim* dims, int nd, int max_naux, int max_pairs, int max_on, int max_v,
-                      const double* C, const double* eps, void* half, double* part, double* E2, cudaStream_t s);
+// else FP32 (energy epilogue on FP32 pairs, FP64 sums).  half: scratch of the
+// half-transformed blocks; part: 2 doubles per occupied pair.
+cudaError_t launch_df(bool fp64, const DfDim* dims, int nd, const DfMax& m, const double* C, const double* eps,
+                      void* half, double* part, double* E2, int sms, cudaStream_t s);
 
 // Split dimers: E2[dimer] = sum, in block order, of E2[first .. first+n) for
 // each (dimer, first, n) triple of `fold` (device, 3 ints each).
