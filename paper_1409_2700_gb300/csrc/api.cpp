@@ -1286,7 +1286,7 @@ static mcpt_status build_plan(mcpt_handle h, mcpt_ctx::Plan& P, int first, int c
         for (int k = b; k < b + nd; k++) max_ao = std::max(max_ao, std::max(P.hDesc[k].nX, P.hDesc[k].nY));
         if (max_ao <= 32) continue;
         std::vector<FinTask> t;
-        finish_tasks(P.hDesc.data() + b, nd, 1 << 22, &t);
+        finish_tasks(P.hDesc.data() + b, nd, 1 << 22, !fp64_data(prec), &t);
         std::vector<int> first(nd);
         for (size_t q = 0; q < t.size(); q++)
             if (t[q].pr0 == 0) first[t[q].dimer] = (int)q;

@@ -86,8 +86,9 @@ struct FinTask {
     int first;            // index of the dimer's first task
     int ntasks;           // tasks of the dimer
 };
-// Split each dimer's pairs into tasks of about `pairs_per_task`.
-void finish_tasks(const DimerDesc* h_desc, int nd, int pairs_per_task, std::vector<FinTask>* out);
+// Split each dimer's pairs into tasks of about `fma_per_task` multiply-adds (by
+// its own sizes alone); fp32: for the mixed forms' kernel.
+void finish_tasks(const DimerDesc* h_desc, int nd, int fma_per_task, bool fp32, std::vector<FinTask>* out);
 
 // How the second half of a wave of monomers of at most 32 AO is dealt out:
 // each dimer's occupied pairs over `parts` CTAs of `warps` (4 or 5) warps.

@@ -645,7 +645,7 @@ k_finish_w32_ff(const DimerDesc* __restrict__ dd, const double* __restrict__ C, 
 // Each GEMM's M x N outputs are cut into 8 x 4 blocks dealt round-robin to the
 // 256 threads, so small and ragged shapes keep the threads on useful work;
 // a thread accumulates its block in registers (per K step 12 loads feed 32
-// FMAs).  H slices and Tm/TmK live in shared memory, the C columns are read
+// FMAs).  FP64 here; the FP32 forms' kernel follows.  H slices and Tm/TmK live in shared memory, the C columns are read
 // through L1.  VA and VKT use the same blocks, so each thread meets its own
 // (a, b) terms for the FP64 epilogue (VA goes through shared memory to free
 // its registers).  One CTA runs a range of pairs of one dimer; its FP64
@@ -653,21 +653,20 @@ k_finish_w32_ff(const DimerDesc* __restrict__ dd, const double* __restrict__ C, 
 constexpr int kTThreads = 256;
 constexpr int kTM = 8, kTN = 4;
 
-template <typename T>
 size_t tiled_smem_bytes(int max_ao)
 {
     const size_t n = (size_t)max_ao;
-    return (n * n + 2 * n * n) * sizeof(T) + 2 * n * (sizeof(double) + sizeof(FF)) + 64;
+    return (n * n + 2 * n * n) * sizeof(double) + 2 * n * sizeof(double) + 64;
 }
 
 // acc[i][j] = sum_k A(m0 + i, k) B(k, n0 + j) over rows < M, columns < N.
-template <typename T, typename FA, typename FB>
-__device__ __forceinline__ void mm_block(T (&acc)[kTM][kTN], int m0, int n0, int M, int N, int K, FA A, FB B)
+template <typename FA, typename FB>
+__device__ __forceinline__ void mm_block(double (&acc)[kTM][kTN], int m0, int n0, int M, int N, int K, FA A, FB B)
 {
 #pragma unroll
     for (int i = 0; i < kTM; i++)
 #pragma unroll
-        for (int j = 0; j < kTN; j++) acc[i][j] = T(0);
+        for (int j = 0; j < kTN; j++) acc[i][j] = 0.0;
     bool mok[kTM], nok[kTN];
 #pragma unroll
     for (int i = 0; i < kTM; i++) mok[i] = m0 + i < M;
@@ -675,11 +674,11 @@ __device__ __forceinline__ void mm_block(T (&acc)[kTM][kTN], int m0, int n0, int
     for (int j = 0; j < kTN; j++) nok[j] = n0 + j < N;
 #pragma unroll 2
     for (int k = 0; k < K; k++) {
-        T a[kTM], b[kTN];
+        double a[kTM], b[kTN];
 #pragma unroll
-        for (int i = 0; i < kTM; i++) a[i] = mok[i] ? A(m0 + i, k) : T(0);
+        for (int i = 0; i < kTM; i++) a[i] = mok[i] ? A(m0 + i, k) : 0.0;
 #pragma unroll
-        for (int j = 0; j < kTN; j++) b[j] = nok[j] ? B(k, n0 + j) : T(0);
+        for (int j = 0; j < kTN; j++) b[j] = nok[j] ? B(k, n0 + j) : 0.0;
 #pragma unroll
         for (int i = 0; i < kTM; i++)
 #pragma unroll
@@ -687,15 +686,14 @@ __device__ __forceinline__ void mm_block(T (&acc)[kTM][kTN], int m0, int n0, int
     }
 }
 
-template <typename T>
-__device__ __forceinline__ void copy_slice(T* S, const T* __restrict__ src, int n, int tid)
+__device__ __forceinline__ void copy_slice(double* S, const double* __restrict__ src, int n, int tid)
 {
     for (int k0 = 0; k0 < n; k0 += 4 * kTThreads) {
-        T v[4];
+        double v[4];
 #pragma unroll
         for (int t = 0; t < 4; t++) {
             const int k = k0 + t * kTThreads + tid;
-            v[t] = k < n ? src[k] : T(0);
+            v[t] = k < n ? src[k] : 0.0;
         }
 #pragma unroll
         for (int t = 0; t < 4; t++) {
@@ -705,40 +703,37 @@ __device__ __forceinline__ void copy_slice(T* S, const T* __restrict__ src, int 
     }
 }
 
-template <typename T, bool PAIRS>
 __global__ void __launch_bounds__(kTThreads, 2)
-k_finish_tiled(const DimerDesc* __restrict__ dd, const FinTask* __restrict__ tasks, const T* __restrict__ C,
-               const double* __restrict__ Epool, const T* __restrict__ H, double* __restrict__ part,
-               int smem_elems, T* __restrict__ VT)
+k_finish_tiled(const DimerDesc* __restrict__ dd, const FinTask* __restrict__ tasks, const double* __restrict__ C,
+               const double* __restrict__ Epool, const double* __restrict__ H, double* __restrict__ part,
+               int smem_elems, double* __restrict__ VT)
 {
     const FinTask tk = tasks[blockIdx.x];
     const DimerDesc& d = dd[tk.dimer];
     const int nX = d.nX, nY = d.nY, oY = d.oY;
     const int vX = d.vX, vY = d.vY;
     const int rows = nX * nY, pairs = d.oX * oY;
-    const T* __restrict__ CXv = C + d.cXv;    // virtual columns
-    const T* __restrict__ CYv = C + d.cYv;
+    const double* __restrict__ CXv = C + d.cXv;    // virtual columns
+    const double* __restrict__ CYv = C + d.cYv;
     const double* eX = Epool + d.eX;          // occupied energies of this block
     const double* eY = Epool + d.eY;
-    const T* H0 = H + d.h_off;
-    const T* H1 = H + d.h_off + (long long)pairs * rows;
+    const double* H0 = H + d.h_off;
+    const double* H1 = H + d.h_off + (long long)pairs * rows;
 
     extern __shared__ __align__(16) unsigned char smraw[];
     double* eXv = reinterpret_cast<double*>(smraw);           // [vX]
     double* eYv = eXv + nX;                                   // [vY]
-    FF* eXs = reinterpret_cast<FF*>(eYv + nY);                // [vX]: e_a as FP32 pairs
-    FF* eYs = eXs + nX;                                       // [vY]
-    T* base = reinterpret_cast<T*>(eYs + nY);
+    double* base = eYv + nY;
     // a group of np pairs runs each phase together (one barrier per phase for
     // the group): as many as the launch's shared memory holds
     const int per_pair = rows + nX * vY + nY * vX;
     const int gmax = max(1, min(tk.pr1 - tk.pr0, smem_elems / per_pair));
-    T* S = base;                                              // H slices [np][rows], then VA [np][vX][vY]
-    T* Tm = S + gmax * rows;                                  // [np][nX][vY]
-    T* TmK = Tm + gmax * nX * vY;                             // [np][nY][vX]
+    double* S = base;                                              // H slices [np][rows], then VA [np][vX][vY]
+    double* Tm = S + gmax * rows;                                  // [np][nX][vY]
+    double* TmK = Tm + gmax * nX * vY;                             // [np][nY][vX]
     const int tid = threadIdx.x;
-    for (int k = tid; k < vX; k += kTThreads) { eXv[k] = Epool[d.eXv + k]; eXs[k] = ff_split(eXv[k]); }
-    for (int k = tid; k < vY; k += kTThreads) { eYv[k] = Epool[d.eYv + k]; eYs[k] = ff_split(eYv[k]); }
+    for (int k = tid; k < vX; k += kTThreads) eXv[k] = Epool[d.eXv + k];
+    for (int k = tid; k < vY; k += kTThreads) eYv[k] = Epool[d.eYv + k];
     // 8 x 4 output blocks of each GEMM shape, per pair
     const int bn_vY = (vY + kTN - 1) / kTN, bn_vX = (vX + kTN - 1) / kTN;
     const int nb1 = ((nX + kTM - 1) / kTM) * bn_vY;          // Tm
@@ -747,20 +742,20 @@ k_finish_tiled(const DimerDesc* __restrict__ dd, const FinTask* __restrict__ tas
 
     const bool store = VT != nullptr && d.vt_off >= 0;
     const long long mXc = (long long)d.oXt * vX, mYc = (long long)d.oYt * vY;
-    T* const Vst = store ? VT + d.vt_off : nullptr;
+    double* const Vst = store ? VT + d.vt_off : nullptr;
     double ej = 0.0, ek = 0.0;
     for (int g0 = tk.pr0; g0 < tk.pr1; g0 += gmax) {
         const int np = min(gmax, tk.pr1 - g0);
-        T acc[kTM][kTN];
+        double acc[kTM][kTN];
         // ---- Tm = H0 C_Y(virtual), every pair of the group
         copy_slice(S, H0 + (long long)g0 * rows, np * rows, tid);
         __syncthreads();
         for (int blk = tid; blk < np * nb1; blk += kTThreads) {
             const int p = blk / nb1, q = blk - p * nb1;
             const int m0 = (q / bn_vY) * kTM, n0 = (q % bn_vY) * kTN;
-            const T* Sp = S + p * rows;
-            T* Tp = Tm + p * nX * vY;
-            mm_block<T>(acc, m0, n0, nX, vY, nY, [&](int m, int k) { return Sp[m * nY + k]; },
+            const double* Sp = S + p * rows;
+            double* Tp = Tm + p * nX * vY;
+            mm_block(acc, m0, n0, nX, vY, nY, [&](int m, int k) { return Sp[m * nY + k]; },
                         [&](int k, int n) { return __ldg(CYv + k * nY + n); });
 #pragma unroll
             for (int a = 0; a < kTM; a++)
@@ -775,9 +770,9 @@ k_finish_tiled(const DimerDesc* __restrict__ dd, const FinTask* __restrict__ tas
         for (int blk = tid; blk < np * nb3; blk += kTThreads) {
             const int p = blk / nb3, q = blk - p * nb3;
             const int m0 = (q / bn_vX) * kTM, n0 = (q % bn_vX) * kTN;
-            const T* Sp = S + p * rows;
-            T* Kp = TmK + p * nY * vX;
-            mm_block<T>(acc, m0, n0, nY, vX, nX, [&](int m, int k) { return Sp[m * nX + k]; },
+            const double* Sp = S + p * rows;
+            double* Kp = TmK + p * nY * vX;
+            mm_block(acc, m0, n0, nY, vX, nX, [&](int m, int k) { return Sp[m * nX + k]; },
                         [&](int k, int n) { return __ldg(CXv + k * nX + n); });
 #pragma unroll
             for (int a = 0; a < kTM; a++)
@@ -792,39 +787,28 @@ k_finish_tiled(const DimerDesc* __restrict__ dd, const FinTask* __restrict__ tas
             const int m0 = (q / bn_vY) * kTM, n0 = (q % bn_vY) * kTN;
             const int pr = g0 + p, i = pr / oY, j = pr - i * oY;
             const double eij = eX[i] + eY[j];
-            const T* Tp = Tm + p * nX * vY;
-            const T* Kp = TmK + p * nY * vX;
-            T* Vp = S + p * rows;                                 // VA of pair p (own elements)
-            mm_block<T>(acc, m0, n0, vX, vY, nX, [&](int m, int k) { return __ldg(CXv + k * nX + m); },
+            const double* Tp = Tm + p * nX * vY;
+            const double* Kp = TmK + p * nY * vX;
+            double* Vp = S + p * rows;                                 // VA of pair p (own elements)
+            mm_block(acc, m0, n0, vX, vY, nX, [&](int m, int k) { return __ldg(CXv + k * nX + m); },
                         [&](int k, int n) { return Tp[k * vY + n]; });
 #pragma unroll
             for (int a = 0; a < kTM; a++)
 #pragma unroll
                 for (int b = 0; b < kTN; b++)
                     if (m0 + a < vX && n0 + b < vY) Vp[(m0 + a) * vY + n0 + b] = acc[a][b];
-            mm_block<T>(acc, m0, n0, vX, vY, nY, [&](int m, int k) { return Kp[k * vX + m]; },
+            mm_block(acc, m0, n0, vX, vY, nY, [&](int m, int k) { return Kp[k * vX + m]; },
                         [&](int k, int n) { return __ldg(CYv + k * nY + n); });
-            [[maybe_unused]] const FF eijs = PAIRS ? ff_split(eij) : FF{0.f, 0.f};
-            [[maybe_unused]] FF sj{0.f, 0.f}, sk{0.f, 0.f};   // this block's sums (PAIRS)
 #pragma unroll
             for (int a = 0; a < kTM; a++) {
                 const int m = m0 + a;
-                [[maybe_unused]] FF eijas{0.f, 0.f};
-                if constexpr (PAIRS)
-                    if (m < vX) eijas = ff_sub(eijs, eXs[m]);
 #pragma unroll
                 for (int b = 0; b < kTN; b++) {
                     const int n = n0 + b;
                     if (m < vX && n < vY) {
-                        const T vab = Vp[m * vY + n];
-                        T tv;
-                        if constexpr (PAIRS) {
-                            tv = energy_terms_ff(vab, acc[a][b], eijas, eYs[n], sj, sk);
-                        } else {
-                            double t;
-                            energy_terms<T>(vab, acc[a][b], eij - (eXv[m] + eYv[n]), ej, ek, store ? &t : nullptr);
-                            tv = store ? narrow<T>(t) : T(0);
-                        }
+                        const double vab = Vp[m * vY + n];
+                        double tv;
+                        energy_terms<double>(vab, acc[a][b], eij - (eXv[m] + eYv[n]), ej, ek, store ? &tv : nullptr);
                         if (store) {
                             const long long e =
                                 ((long long)(d.jY0 + j) * vY + n) * mXc + (long long)(d.iX0 + i) * vX + m;
@@ -833,10 +817,6 @@ k_finish_tiled(const DimerDesc* __restrict__ dd, const FinTask* __restrict__ tas
                         }
                     }
                 }
-            }
-            if constexpr (PAIRS) {
-                ej += ff_f64(sj);
-                ek += ff_f64(sk);
             }
         }
         __syncthreads();
@@ -855,21 +835,297 @@ k_finish_tiled(const DimerDesc* __restrict__ dd, const FinTask* __restrict__ tas
     }
 }
 
-// Per dimer: its task partials in task order -> {4 sum, -2 sum}.
-__global__ void k_finish_sum(const DimerDesc* __restrict__ dd, int nd, const FinTask* __restrict__ tasks,
-                             const int* __restrict__ first_task, const double* __restrict__ part,
-                             double* __restrict__ E2)
+// FP32 (mixed forms).  The same four products on 8 x 8 blocks, two columns per
+// packed multiply-add, every operand in shared memory: both virtual coefficient
+// blocks for the whole task, the pairs' H slices, and Tm / TmK in the slices'
+// place (written from registers once the slice is consumed).  A thread has one
+// block of each product -- as many pairs as fill 256 threads run together --
+// and keeps its (ia|jb) block in registers until it meets (ib|ja) in the
+// epilogue.  A second set of slices, where it fits, is filled while the first
+// is used.  A block's columns are 4 nb .. 4 nb + 3 and the same in the upper half, so
+// that a warp's 16-byte loads are contiguous.  Every output is one chain over k
+// in order.  Bound by the FP32 pipes at eight warps per SM (64 accumulators
+// twice): 1200 pairs of 128 + 128 AO in 0.63 ms, 25 TFLOP/s; the FP64 kernel's
+// scheme above (8 x 4 blocks, scalar loads, C through L1) took 1.55 ms there in
+// FP32, and 1.41 ms against 0.78 for 96 dimers of 16 to 96 AO.
+constexpr int kF32Cap = 220 * 1024;   // shared bytes a launch may use
+
+struct TiledShape {
+    int bmX, bmY, bnX, bnY;            // 8-blocks of nX, nY, vX, vY
+    int kX, kY;                        // nX, nY padded to 4
+    int np, nbuf, slab;                // pairs of a group, slice sets, elements of a pair's slice
+    int c_elems;
+};
+
+// The shape for a dimer within `elems` shared floats.
+__host__ __device__ inline TiledShape tiled_shape(int nX, int nY, int vX, int vY, int elems)
 {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= nd) return;
-    const FinTask t0 = tasks[first_task[k]];
-    double sj = 0.0, sk = 0.0;
-    for (int t = t0.first; t < t0.first + t0.ntasks; t++) {
-        sj += part[2 * t];
-        sk += part[2 * t + 1];
+    TiledShape t;
+    t.bmX = (nX + 7) / 8; t.bmY = (nY + 7) / 8; t.bnX = (vX + 7) / 8; t.bnY = (vY + 7) / 8;
+    t.kX = (nX + 3) / 4 * 4; t.kY = (nY + 3) / 4 * 4;
+    const int rX = 8 * t.bmX * (t.kY + 4 > 8 * t.bnY ? t.kY + 4 : 8 * t.bnY);
+    const int rY = 8 * t.bmY * (t.kX + 4 > 8 * t.bnX ? t.kX + 4 : 8 * t.bnX);
+    t.slab = rX > rY ? rX : rY;
+    t.c_elems = t.kX * 8 * t.bnX + t.kY * 8 * t.bnY;
+    int nb = t.bmX * t.bnY;
+    if (t.bmY * t.bnX > nb) nb = t.bmY * t.bnX;
+    t.np = kTThreads / nb;
+    const int fit = (elems - t.c_elems) / t.slab;
+    if (t.np > fit) t.np = fit;
+    t.nbuf = 2 * t.np <= fit ? 2 : 1;
+    return t;
+}
+
+// Copy np slices (rows x cols, contiguous, `rows * cols` apart) into
+// S[p][up8(rows)][ld], zero beyond the rows and columns (up to colsp), by cp.async.
+__device__ __forceinline__ void load_slices(float* S, const float* __restrict__ src, int np, int rows, int cols,
+                                            int rowsp, int colsp, int ld, int slab, int tid)
+{
+    if ((cols & 3) == 0 && ((size_t)src & 15) == 0) {
+        const int pc = cols / 4, per = rowsp * pc;
+        for (int e = tid; e < np * per; e += kTThreads) {
+            const int p = e / per, r = (e - p * per) / pc, c = (e - p * per - r * pc) * 4;
+            const bool ok = r < rows;
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(
+                             (unsigned)__cvta_generic_to_shared(S + p * slab + r * ld + c)),
+                         "l"(ok ? src + ((long long)p * rows + r) * cols + c : src), "r"(ok ? 16 : 0)
+                         : "memory");
+        }
+    } else {
+        const int per = rowsp * colsp;
+        for (int e = tid; e < np * per; e += kTThreads) {
+            const int p = e / per, r = (e - p * per) / colsp, c = e - p * per - r * colsp;
+            const bool ok = r < rows && c < cols;
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(
+                             (unsigned)__cvta_generic_to_shared(S + p * slab + r * ld + c)),
+                         "l"(ok ? src + ((long long)p * rows + r) * cols + c : src), "r"(ok ? 4 : 0)
+                         : "memory");
+        }
     }
-    E2[2 * dd[k].slot + 0] = 4.0 * sj;
-    E2[2 * dd[k].slot + 1] = -2.0 * sk;
+    asm volatile("cp.async.commit_group;" ::: "memory");
+}
+
+__device__ __forceinline__ void zero8(float2 (&acc)[8][4])
+{
+#pragma unroll
+    for (int i = 0; i < 8; i++)
+#pragma unroll
+        for (int j = 0; j < 4; j++) acc[i][j] = make_float2(0.f, 0.f);
+}
+
+// acc[i] += a[i] b, b the block's eight columns.
+__device__ __forceinline__ void outer8(float2 (&acc)[8][4], const float (&a)[8], const float* b, int half)
+{
+    const float4 lo = *reinterpret_cast<const float4*>(b), hi = *reinterpret_cast<const float4*>(b + half);
+#pragma unroll
+    for (int i = 0; i < 8; i++) {
+        const float2 x = make_float2(a[i], a[i]);
+        acc[i][0] = __ffma2_rn(x, make_float2(lo.x, lo.y), acc[i][0]);
+        acc[i][1] = __ffma2_rn(x, make_float2(lo.z, lo.w), acc[i][1]);
+        acc[i][2] = __ffma2_rn(x, make_float2(hi.x, hi.y), acc[i][2]);
+        acc[i][3] = __ffma2_rn(x, make_float2(hi.z, hi.w), acc[i][3]);
+    }
+}
+
+// acc = sum_k A[i][k] B[k][.], A row-major (four k per 16-byte load), K a multiple of 4.
+__device__ __forceinline__ void mm_rows(float2 (&acc)[8][4], const float* A, int lda, const float* B, int ldb, int K)
+{
+    zero8(acc);
+#pragma unroll 1
+    for (int k = 0; k < K; k += 4) {
+        float4 a[8];
+#pragma unroll
+        for (int i = 0; i < 8; i++) a[i] = *reinterpret_cast<const float4*>(A + i * lda + k);
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+            float x[8];
+#pragma unroll
+            for (int i = 0; i < 8; i++) x[i] = u == 0 ? a[i].x : u == 1 ? a[i].y : u == 2 ? a[i].z : a[i].w;
+            outer8(acc, x, B + (k + u) * ldb, ldb / 2);
+        }
+    }
+}
+
+// acc = sum_k A[k][i] B[k][.], both k-major.
+__device__ __forceinline__ void mm_cols(float2 (&acc)[8][4], const float* A, int lda, const float* B, int ldb, int K)
+{
+    zero8(acc);
+#pragma unroll 2
+    for (int k = 0; k < K; k++) {
+        const float4 p = *reinterpret_cast<const float4*>(A + k * lda), q = *reinterpret_cast<const float4*>(A + k * lda + 4);
+        const float x[8] = {p.x, p.y, p.z, p.w, q.x, q.y, q.z, q.w};
+        outer8(acc, x, B + k * ldb, ldb / 2);
+    }
+}
+
+__device__ __forceinline__ void put8(float* T, int ld, const float2 (&acc)[8][4])
+{
+#pragma unroll
+    for (int i = 0; i < 8; i++) {
+        *reinterpret_cast<float4*>(T + i * ld) = make_float4(acc[i][0].x, acc[i][0].y, acc[i][1].x, acc[i][1].y);
+        *reinterpret_cast<float4*>(T + i * ld + ld / 2) = make_float4(acc[i][2].x, acc[i][2].y, acc[i][3].x, acc[i][3].y);
+    }
+}
+
+template <bool PAIRS>
+__global__ void __launch_bounds__(kTThreads, 1)
+k_finish_tiled_f32(const DimerDesc* __restrict__ dd, const FinTask* __restrict__ tasks, const float* __restrict__ C,
+                   const double* __restrict__ Epool, const float* __restrict__ H, double* __restrict__ part,
+                   int smem_elems, float* __restrict__ VT)
+{
+    const FinTask tk = tasks[blockIdx.x];
+    const DimerDesc& d = dd[tk.dimer];
+    const int nX = d.nX, nY = d.nY, oY = d.oY, vX = d.vX, vY = d.vY;
+    const int rows = nX * nY, pairs = d.oX * oY;
+    const TiledShape t = tiled_shape(nX, nY, vX, vY, smem_elems);
+    const int vX8 = 8 * t.bnX, vY8 = 8 * t.bnY, ldY = t.kY + 4, ldX = t.kX + 4;
+    const float* H0 = H + d.h_off;
+    const float* H1 = H0 + (long long)pairs * rows;
+    extern __shared__ __align__(16) unsigned char smraw[];
+    float* sCX = reinterpret_cast<float*>(smraw);              // [kX][vX8], zero padded
+    float* sCY = sCX + t.kX * vX8;                             // [kY][vY8]
+    float* S0 = sCY + t.kY * vY8;
+    float* S1 = t.nbuf == 2 ? S0 + t.np * t.slab : S0;
+    const int tid = threadIdx.x;
+    for (int e = tid; e < t.c_elems; e += kTThreads) {
+        const bool y = e >= t.kX * vX8;
+        const int f = y ? e - t.kX * vX8 : e, w = y ? vY8 : vX8, n = y ? nY : nX, k = f / w, c = f - k * w;
+        const bool ok = k < n && c < (y ? vY : vX);
+        const float* src = C + (y ? d.cYv : d.cXv);
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"((unsigned)__cvta_generic_to_shared(sCX + e)),
+                     "l"(ok ? src + k * n + c : src), "r"(ok ? 4 : 0)
+                     : "memory");
+    }
+    load_slices(S0, H0 + (long long)tk.pr0 * rows, min(t.np, tk.pr1 - tk.pr0), nX, nY, 8 * t.bmX, t.kY, ldY, t.slab, tid);
+    const int nb1 = t.bmX * t.bnY, nb3 = t.bmY * t.bnX, nb2 = t.bnX * t.bnY;
+    // this thread's block of each product: pair p, row block m, column block n
+    const int p1 = tid / nb1, m1 = (tid - p1 * nb1) / t.bnY, n1 = tid - p1 * nb1 - m1 * t.bnY;
+    const int p3 = tid / nb3, m3 = (tid - p3 * nb3) / t.bnX, n3 = tid - p3 * nb3 - m3 * t.bnX;
+    const int p2 = tid / nb2, m2 = (tid - p2 * nb2) / t.bnY, n2 = tid - p2 * nb2 - m2 * t.bnY;
+    const bool store = VT != nullptr && d.vt_off >= 0;
+    const long long mXc = (long long)d.oXt * vX, mYc = (long long)d.oYt * vY;
+    float* const Vst = store ? VT + d.vt_off : nullptr;
+    double ej = 0.0, ek = 0.0;
+    for (int g0 = tk.pr0; g0 < tk.pr1; g0 += t.np) {
+        const int np = min(t.np, tk.pr1 - g0);
+        float2 acc[8][4], v[8][4];
+        if (t.nbuf == 2) {
+            load_slices(S1, H1 + (long long)g0 * rows, np, nY, nX, 8 * t.bmY, t.kX, ldX, t.slab, tid);
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+        } else {
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+        }
+        __syncthreads();
+        // ---- Tm[nu][b] = sum_sig H0[nu][sig] C_Y[sig][b], then in the slice's place
+        if (p1 < np) mm_rows(acc, S0 + p1 * t.slab + 8 * m1 * ldY, ldY, sCY + 4 * n1, vY8, t.kY);
+        __syncthreads();
+        if (p1 < np) put8(S0 + p1 * t.slab + 8 * m1 * vY8 + 4 * n1, vY8, acc);
+        __syncthreads();
+        // ---- (ia|jb) = sum_nu C_X[nu][a] Tm[nu][b]
+        if (p2 < np) mm_cols(v, sCX + 8 * m2, vX8, S0 + p2 * t.slab + 4 * n2, vY8, t.kX);
+        __syncthreads();
+        const int nn = min(t.np, tk.pr1 - g0 - t.np);   // the next group's pairs
+        if (t.nbuf == 1) {
+            load_slices(S1, H1 + (long long)g0 * rows, np, nY, nX, 8 * t.bmY, t.kX, ldX, t.slab, tid);
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+        } else if (nn > 0) {
+            load_slices(S0, H0 + (long long)(g0 + t.np) * rows, nn, nX, nY, 8 * t.bmX, t.kY, ldY, t.slab, tid);
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+        } else {
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+        }
+        __syncthreads();
+        // ---- TmK[lam][a] = sum_nu H1[lam][nu] C_X[nu][a]
+        if (p3 < np) mm_rows(acc, S1 + p3 * t.slab + 8 * m3 * ldX, ldX, sCX + 4 * n3, vX8, t.kX);
+        __syncthreads();
+        if (p3 < np) put8(S1 + p3 * t.slab + 8 * m3 * vX8 + 4 * n3, vX8, acc);
+        __syncthreads();
+        // ---- (ib|ja) = sum_lam TmK[lam][a] C_Y[lam][b], and the epilogue
+        if (p2 < np) {
+            mm_cols(acc, S1 + p2 * t.slab + 8 * m2, vX8, sCY + 4 * n2, vY8, t.kY);
+            const int pr = g0 + p2, i = pr / oY, j = pr - i * oY;
+            const double eij = Epool[d.eX + i] + Epool[d.eY + j];
+            const int b0 = 4 * n2, b1 = b0 + vY8 / 2;
+            [[maybe_unused]] FF sj{0.f, 0.f}, sk{0.f, 0.f}, ebs[8];
+            [[maybe_unused]] const FF eijs = ff_split(eij);
+            if constexpr (PAIRS) {
+#pragma unroll
+                for (int c = 0; c < 8; c++) {
+                    const int b = (c < 4 ? b0 : b1 - 4) + c;
+                    ebs[c] = b < vY ? ff_split(Epool[d.eYv + b]) : FF{0.f, 0.f};
+                }
+            }
+#pragma unroll
+            for (int r = 0; r < 8; r++) {
+                const int a = 8 * m2 + r;
+                if (a >= vX) break;
+                const double ea = Epool[d.eXv + a];
+                [[maybe_unused]] FF eijas{0.f, 0.f};
+                if constexpr (PAIRS) eijas = ff_sub(eijs, ff_split(ea));
+#pragma unroll
+                for (int c = 0; c < 8; c++) {
+                    const int b = (c < 4 ? b0 : b1 - 4) + c;
+                    if (b < vY) {
+                        const float vab = c & 1 ? v[r][c / 2].y : v[r][c / 2].x;
+                        const float vk = c & 1 ? acc[r][c / 2].y : acc[r][c / 2].x;
+                        float tv;
+                        if constexpr (PAIRS) {
+                            tv = energy_terms_ff(vab, vk, eijas, ebs[c], sj, sk);
+                        } else {
+                            double x;
+                            energy_terms<float>(vab, vk, eij - (ea + Epool[d.eYv + b]), ej, ek, store ? &x : nullptr);
+                            tv = store ? narrow<float>(x) : 0.f;
+                        }
+                        if (store) {
+                            const long long e = ((long long)(d.jY0 + j) * vY + b) * mXc + (long long)(d.iX0 + i) * vX + a;
+                            Vst[e] = vab;
+                            Vst[mXc * mYc + e] = tv;
+                        }
+                    }
+                }
+            }
+            if constexpr (PAIRS) {
+                ej += ff_f64(sj);
+                ek += ff_f64(sk);
+            }
+        }
+        if (t.nbuf == 1 && nn > 0) {
+            __syncthreads();
+            load_slices(S0, H0 + (long long)(g0 + t.np) * rows, nn, nX, nY, 8 * t.bmX, t.kY, ldY, t.slab, tid);
+        } else {
+            __syncthreads();                     // S1 consumed before the next group's H1
+        }
+    }
+    // fixed-order block reduction
+    __shared__ double red[2][kTThreads / 32];
+    ej = warp_sum(ej);
+    ek = warp_sum(ek);
+    if ((tid & 31) == 0) { red[0][tid >> 5] = ej; red[1][tid >> 5] = ek; }
+    __syncthreads();
+    if (tid == 0) {
+        double sj = 0.0, sk = 0.0;
+        for (int w = 0; w < kTThreads / 32; w++) { sj += red[0][w]; sk += red[1][w]; }
+        part[2 * blockIdx.x + 0] = sj;
+        part[2 * blockIdx.x + 1] = sk;
+    }
+}
+
+// Per dimer: its task partials -> {4 sum, -2 sum}; a warp each, lane l tasks l,
+// l + 32, ... in order, then the fixed tree (400 tasks of a 128-AO dimer added
+// by one thread took 23 to 40 us).
+__global__ void __launch_bounds__(32)
+k_finish_sum(const DimerDesc* __restrict__ dd, const FinTask* __restrict__ tasks, const int* __restrict__ first_task,
+             const double* __restrict__ part, double* __restrict__ E2)
+{
+    const int k = blockIdx.x, lane = threadIdx.x;
+    const FinTask t0 = tasks[first_task[k]];
+    double ej = 0.0, ek = 0.0;
+    for (int t = t0.first + lane; t < t0.first + t0.ntasks; t += 32) {
+        ej += part[2 * t];
+        ek += part[2 * t + 1];
+    }
+    const double s = pair_tree(ej, ek, lane);
+    if ((lane & 15) == 0) E2[2 * dd[k].slot + (lane >> 4)] = lane ? -2.0 * s : 4.0 * s;
 }
 
 template <typename T, bool PAIRS, int W>
@@ -898,16 +1154,24 @@ cudaError_t launch_finish(const DimerDesc* d_desc, int nd, int max_ao, const T* 
         return sp.warps == 5 ? launch_w32<T, PAIRS, 5>(d_desc, nd, C, Epool, H, E2, VT, sp, s)
                              : launch_w32<T, PAIRS, 4>(d_desc, nd, C, Epool, H, E2, VT, sp, s);
     if (!tasks || ntasks <= 0 || !part) return cudaErrorInvalidValue;
-    const size_t smem = tiled_smem_bytes<T>(max_ao);
-    if (smem > 227 * 1024) return cudaErrorInvalidValue;
-    cudaError_t e = cudaFuncSetAttribute(k_finish_tiled<T, PAIRS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    const int smem_elems = (int)((smem - 2 * max_ao * (sizeof(double) + sizeof(FF)) - 64) / sizeof(T));
-    k_finish_tiled<T, PAIRS><<<ntasks, kTThreads, smem, s>>>(d_desc, tasks, C, Epool, H, part, smem_elems, VT);
+    cudaError_t e;
+    if constexpr (sizeof(T) == 4) {
+        e = cudaFuncSetAttribute(k_finish_tiled_f32<PAIRS>, cudaFuncAttributeMaxDynamicSharedMemorySize, kF32Cap);
+        if (e != cudaSuccess) return e;
+        k_finish_tiled_f32<PAIRS><<<ntasks, kTThreads, kF32Cap, s>>>(d_desc, tasks, C, Epool, H, part,
+                                                                      kF32Cap / (int)sizeof(float), VT);
+    } else {
+        const size_t smem = tiled_smem_bytes(max_ao);
+        if (smem > 227 * 1024) return cudaErrorInvalidValue;
+        e = cudaFuncSetAttribute(k_finish_tiled, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        const int smem_elems = (int)((smem - 2 * max_ao * sizeof(double) - 64) / sizeof(double));
+        k_finish_tiled<<<ntasks, kTThreads, smem, s>>>(d_desc, tasks, C, Epool, H, part, smem_elems, VT);
+    }
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     // the dimers' first-task indices follow the task array
     const int* first = reinterpret_cast<const int*>(tasks + ntasks);
-    k_finish_sum<<<(nd + 127) / 128, 128, 0, s>>>(d_desc, nd, tasks, first, part, E2);
+    k_finish_sum<<<nd, 32, 0, s>>>(d_desc, tasks, first, part, E2);
     return cudaGetLastError();
 }
 
@@ -1112,14 +1376,17 @@ FinSplit finish_w32_split(const DimerDesc* h, int nd, int form, int sms)
     return five ? FinSplit{5, p5, nullptr} : FinSplit{4, p4, nullptr};
 }
 
-void finish_tasks(const DimerDesc* h, int nd, int fma_per_task, std::vector<FinTask>* out)
+void finish_tasks(const DimerDesc* h, int nd, int fma_per_task, bool fp32, std::vector<FinTask>* out)
 {
     out->clear();
     for (int k = 0; k < nd; k++) {
         const long long nX = h[k].nX, nY = h[k].nY, vX = h[k].vX, vY = h[k].vY;
         const int pairs = h[k].oX * h[k].oY;
         const long long per_pair = 2 * (nX * nY * vY + vX * vY * nX);   // FMAs of one pair, both forms
-        const int ppt = (int)std::max<long long>(1, std::min<long long>(pairs, fma_per_task / std::max(1LL, per_pair)));
+        // FP32: whole groups of the pairs that run together
+        const int grp = !fp32 ? 1 : tiled_shape((int)nX, (int)nY, (int)vX, (int)vY, kF32Cap / (int)sizeof(float)).np;
+        const int ppt = (int)std::max<long long>(1, std::min<long long>((pairs + grp - 1) / grp,
+                                                                        fma_per_task / std::max(1LL, per_pair * grp))) * grp;
         const int ntasks = (pairs + ppt - 1) / ppt;
         const int first = (int)out->size();
         for (int t = 0; t < ntasks; t++)
