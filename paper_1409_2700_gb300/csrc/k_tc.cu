@@ -47,6 +47,7 @@ namespace mcpt {
 struct TcItem {
     int dimer;   // index within the launch's descriptor array
     int form;    // 0: A block, 1: K block
+    int p1t;     // p1 values per M-tile (tile_p1)
     int mt0;     // first M-tile
     int mts;     // number of M-tiles (accumulators) in this item
 };
@@ -354,7 +355,7 @@ struct ItemGeo {
     int rows;         // n1 * n3
 };
 
-__device__ __forceinline__ ItemGeo geo_of(const DimerDesc& d, int f)
+__device__ __forceinline__ ItemGeo geo_of(const DimerDesc& d, int f, int p1t)
 {
     ItemGeo g;
     g.n0 = d.nX;
@@ -363,7 +364,7 @@ __device__ __forceinline__ ItemGeo geo_of(const DimerDesc& d, int f)
     g.n3 = f ? d.nX : d.nY;
     g.o0 = d.oX;
     g.o2 = d.oY;
-    g.p1t = 128 / g.n3;
+    g.p1t = p1t;
     g.kcs = (g.n2 + kKC - 1) / kKC;
     g.kblocks = g.n0 * g.kcs;
     g.N = d.npad;
@@ -461,7 +462,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_half_tc(const TcParams P)
             for (int it = blockIdx.x; it < P.n_items && !sh->abort; it += gridDim.x) {
                 const TcItem item = P.items[it];
                 const DimerDesc& d = P.desc[item.dimer];
-                const ItemGeo g = geo_of(d, item.form);
+                const ItemGeo g = geo_of(d, item.form, item.p1t);
                 const CUtensorMap* map = P.maps + 2 * item.dimer + item.form;
                 const unsigned box = (unsigned)g.n3 * kKC * g.p1t * 8u;
                 for (int kb = 0; kb < g.kblocks && !sh->abort; kb++) {
@@ -492,7 +493,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_half_tc(const TcParams P)
             bool any = false;
             for (int it = blockIdx.x; it < P.n_items && !sh->abort; it += gridDim.x, li++) {
                 const TcItem item = P.items[it];
-                const ItemGeo g = geo_of(P.desc[item.dimer], item.form);
+                const ItemGeo g = geo_of(P.desc[item.dimer], item.form, item.p1t);
                 const unsigned idesc = make_idesc(KIND, g.N);
                 const int b = li & 1;
                 if (!mbar_wait(&sh->tmem_empty[b], ((li >> 1) & 1) ^ 1, &sh->abort, P.status, 2, P.wait_ns)) break;
@@ -544,7 +545,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_half_tc(const TcParams P)
         for (int it = blockIdx.x; it < P.n_items && !sh->abort; it += gridDim.x) {
             const TcItem item = P.items[it];
             const DimerDesc& d = P.desc[item.dimer];
-            const ItemGeo g = geo_of(d, item.form);
+            const ItemGeo g = geo_of(d, item.form, item.p1t);
             const float* CX = P.Cf + d.cX;
             const float* CY = P.Cf + d.cY;
             const int npairs = g.o0 * g.o2;
@@ -667,7 +668,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_half_tc(const TcParams P)
         for (int it = blockIdx.x; it < P.n_items && !sh->abort; it += gridDim.x, li++) {
             const TcItem item = P.items[it];
             const DimerDesc& d = P.desc[item.dimer];
-            const ItemGeo g = geo_of(d, item.form);
+            const ItemGeo g = geo_of(d, item.form, item.p1t);
             const int b = li & 1;
             if (!mbar_wait(&sh->tmem_full[b], (li >> 1) & 1, &sh->abort, P.status, 8, P.wait_ns)) break;
             tc_fence_after();
@@ -1425,7 +1426,7 @@ __global__ void __launch_bounds__(rank_threads<BIG, OB, KIND>(), 1) k_half_tc_ra
             bool ok = true;
             for (int it = blockIdx.x; it < P.n_items && ok && !*abort; it += gridDim.x) {
                 const TcItem item = P.items[it];
-                const ItemGeo g = geo_of(P.desc[item.dimer], item.form);
+                const ItemGeo g = geo_of(P.desc[item.dimer], item.form, item.p1t);
                 const CUtensorMap* map = P.maps + 2 * item.dimer + item.form;
                 const unsigned box = (unsigned)g.n3 * kKC * g.p1t * 8u;
                 for (int mt = 0; mt < item.mts && ok; mt++)
@@ -1465,7 +1466,7 @@ __global__ void __launch_bounds__(rank_threads<BIG, OB, KIND>(), 1) k_half_tc_ra
             for (int u = 0; u < 6; u++) idesc_f6[u] = make_idesc(KIND, (7 - u) * kNT);
             for (int it = blockIdx.x; it < P.n_items && ok && !*abort; it += gridDim.x, li++) {
                 const TcItem item = P.items[it];
-                const ItemGeo g = geo_of(P.desc[item.dimer], item.form);
+                const ItemGeo g = geo_of(P.desc[item.dimer], item.form, item.p1t);
                 const int wp = li & 1;
                 if (!(ok = mbar_wait(&sh->full_w[wp], (li >> 1) & 1, abort, P.status, 12, P.wait_ns))) break;
                 for (int mt = 0; mt < item.mts && ok; mt++)
@@ -1570,7 +1571,7 @@ __global__ void __launch_bounds__(rank_threads<BIG, OB, KIND>(), 1) k_half_tc_ra
         for (int it = blockIdx.x; it < P.n_items && ok && !*abort; it += gridDim.x, li++) {
             const TcItem item = P.items[it];
             const DimerDesc& d = P.desc[item.dimer];
-            const ItemGeo g = geo_of(d, item.form);
+            const ItemGeo g = geo_of(d, item.form, item.p1t);
             const float* CY = P.Cf + d.cY;
             [[maybe_unused]] const double* CYd = P.Cd + d.cY;   // FP64E: C_Y in FP64
             const int wp = li & 1;
@@ -1764,7 +1765,7 @@ __global__ void __launch_bounds__(rank_threads<BIG, OB, KIND>(), 1) k_half_tc_ra
         for (int it = blockIdx.x; it < P.n_items && ok && !*abort; it += gridDim.x, li++) {
             const TcItem item = P.items[it];
             const DimerDesc& d = P.desc[item.dimer];
-            const ItemGeo g = geo_of(d, item.form);
+            const ItemGeo g = geo_of(d, item.form, item.p1t);
             const int par = li & 1;
             float* cx = cxs + par * CXF;
             // stage C_X's occupied columns, row p0 = e, for this item
@@ -1976,10 +1977,13 @@ PFN_cuTensorMapEncodeTiled_v12000 get_encode()
 
 // The rank variants (1-3) run one M-tile per item; variant 0 groups as many
 // M-tiles as one TMEM accumulator set holds.
-int items_per_form(const DimerDesc& d, int f, int variant, int* mts_max)
+// p1 values per M-tile: as many as fill its 128 rows, or a `split` of that.
+int tile_p1(int n3, int split) { return std::max(1, 128 / n3 / split); }
+
+int items_per_form(const DimerDesc& d, int f, int variant, int split, int* mts_max)
 {
     const int n1 = f ? d.nY : d.nX, n3 = f ? d.nX : d.nY;
-    const int p1t = 128 / n3;
+    const int p1t = tile_p1(n3, split);
     const int tiles = (n1 + p1t - 1) / p1t;
     const int mmax = variant >= 1 ? 1 : std::max(1, std::min(8, kAccCols / d.npad));
     *mts_max = mmax;
@@ -2014,16 +2018,43 @@ int choose_variant(TcKind kind, const DimerDesc* h, int nd)
     return omax <= kOB5 ? 3 : omax <= kOB ? 1 : 2;
 }
 
+// A wave whose full tiles are fewer than the SMs (one item each) takes
+// smaller ones: the largest split that still gives each SM at most one item.
+// One dimer of 32 AO, first half: BF16x2 30 -> 26 us, BF16x3 41 -> 31, FP64E 76 ->
+// 62; one of 48 AO in BF16x2 86 -> 76.  Beyond one item per SM it only adds
+// units that convert fewer rows each: six dimers 32 -> 49 us.  Rows do not
+// share anything, so the results are the same bits.
+int tile_split(const DimerDesc* h, int nd, int variant)
+{
+    if (variant == 0) return 1;
+    int dev = 0, nsm = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    int split = 1;
+    for (int s = 2; s <= 64; s *= 2) {
+        long long items = 0;
+        for (int k = 0; k < nd && items <= nsm; k++)
+            for (int f = 0; f < 2; f++) {
+                int m;
+                items += items_per_form(h[k], f, variant, s, &m);
+            }
+        if (items > nsm) break;
+        split = s;
+    }
+    return split;
+}
+
 }  // namespace
 
 size_t tc_work_bytes(TcKind kind, const DimerDesc* h, int nd)
 {
     size_t items = 0;
     const int variant = choose_variant(kind, h, nd);
+    const int split = tile_split(h, nd, 1);   // the same for every rank kernel; no fewer items than others
     for (int k = 0; k < nd; k++)
         for (int f = 0; f < 2; f++) {
             int m;
-            items += items_per_form(h[k], f, variant, &m);
+            items += items_per_form(h[k], f, variant, split, &m);
         }
     return (size_t)nd * 2 * sizeof(CUtensorMap) + items * sizeof(TcItem) + 256;
 }
@@ -2122,12 +2153,13 @@ cudaError_t tc_prepare(TcKind kind, const DimerDesc* h_desc, const DimerDesc* d_
     }
     int maxN = 16;
     unsigned max_box = 0;
+    const int split = tile_split(h_desc, nd, variant);
     for (int k = 0; k < nd; k++) {
         const DimerDesc& d = h_desc[k];
         maxN = std::max(maxN, d.npad);
         for (int f = 0; f < 2; f++) {
             const int n0 = d.nX, n1 = f ? d.nY : d.nX, n2 = d.nY, n3 = f ? d.nX : d.nY;
-            const int p1t = 128 / n3;
+            const int p1t = tile_p1(n3, split);
             cuuint64_t dims[4] = {(cuuint64_t)n3, (cuuint64_t)n2, (cuuint64_t)n1, (cuuint64_t)n0};
             cuuint64_t strides[3] = {(cuuint64_t)d.st[f][2] * 8, (cuuint64_t)d.st[f][1] * 8, (cuuint64_t)d.st[f][0] * 8};
             cuuint32_t box[4] = {(cuuint32_t)n3, (cuuint32_t)kKC, (cuuint32_t)p1t, 1};
@@ -2141,12 +2173,13 @@ cudaError_t tc_prepare(TcKind kind, const DimerDesc* h_desc, const DimerDesc* d_
             }
             max_box = std::max(max_box, (unsigned)(n3 * kKC * p1t * 8));
             int mmax;
-            const int nit = items_per_form(d, f, variant, &mmax);
+            const int nit = items_per_form(d, f, variant, split, &mmax);
             const int tiles = (n1 + p1t - 1) / p1t;
             for (int q = 0; q < nit; q++) {
                 TcItem it;
                 it.dimer = k;
                 it.form = f;
+                it.p1t = p1t;
                 it.mt0 = q * mmax;
                 it.mts = std::min(mmax, tiles - it.mt0);
                 items.push_back(it);
