@@ -1286,7 +1286,7 @@ static mcpt_status build_plan(mcpt_handle h, mcpt_ctx::Plan& P, int first, int c
         for (int k = b; k < b + nd; k++) max_ao = std::max(max_ao, std::max(P.hDesc[k].nX, P.hDesc[k].nY));
         if (max_ao <= 32) continue;
         std::vector<FinTask> t;
-        finish_tasks(P.hDesc.data() + b, nd, 1 << 22, !fp64_data(prec), &t);
+        const int nparts = finish_tasks(P.hDesc.data() + b, nd, !fp64_data(prec), h->sms, &t);
         std::vector<int> first(nd);
         for (size_t q = 0; q < t.size(); q++)
             if (t[q].pr0 == 0) first[t[q].dimer] = (int)q;
@@ -1298,7 +1298,7 @@ static mcpt_status build_plan(mcpt_handle h, mcpt_ctx::Plan& P, int first, int c
         std::memcpy(fin_host.data() + fin_off[w] + tb, first.data(), fb);
         ntasks[w] = (int)t.size();
         part_off[w] = parts;
-        parts += t.size();
+        parts += nparts;
     }
     if (!fin_host.empty()) {
         if ((st = ensure(h, &P.dFin, &P.capFin, fin_host.size()))) return st;

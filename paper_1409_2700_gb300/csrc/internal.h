@@ -83,12 +83,12 @@ cudaError_t launch_half_fp32c(const DimerDesc* d_desc, int nd, int max_rows, int
 struct FinTask {
     int dimer;            // descriptor index within the wave
     int pr0, pr1;         // pairs [pr0, pr1) (pair = i*oY + j)
-    int first;            // index of the dimer's first task
-    int ntasks;           // tasks of the dimer
+    int first;            // the dimer's first partial sum
+    int nparts;           // and how many it has: one per task, FP32 one per pair
 };
-// Split each dimer's pairs into tasks of about `fma_per_task` multiply-adds (by
-// its own sizes alone); fp32: for the mixed forms' kernel.
-void finish_tasks(const DimerDesc* h_desc, int nd, int fma_per_task, bool fp32, std::vector<FinTask>* out);
+// Split each dimer's pairs into tasks (fp32: for the mixed forms' kernel, on
+// `sms` SMs); returns the partial sums they write.
+int finish_tasks(const DimerDesc* h_desc, int nd, bool fp32, int sms, std::vector<FinTask>* out);
 
 // How the second half of a wave of monomers of at most 32 AO is dealt out:
 // each dimer's occupied pairs over `parts` CTAs of `warps` (4 or 5) warps.
@@ -102,8 +102,7 @@ struct FinSplit {
 // Second half + denominators + energies.  H is double (FP64 form) or float;
 // waves whose monomers all have <= 32 AO run the split's CTAs, which leave
 // the pairs' sums in H; larger ones run the tasks (`tasks`, device array of
-// `ntasks`) and sum each dimer's task partials (`part`, 2 doubles per task)
-// in task order.
+// `ntasks`) and sum each dimer's partials (`part`, 2 doubles each) in order.
 // With VT non-null, descriptors with vt_off >= 0 also store their (ia|jb)
 // and T = vD for the coupling.  FP32 (mixed forms): the energy epilogue on
 // FP32 pairs, or with fp64_epilogue on the FP64 pipe term by term.

@@ -1005,9 +1005,10 @@ k_finish_tiled_f32(const DimerDesc* __restrict__ dd, const FinTask* __restrict__
     const bool store = VT != nullptr && d.vt_off >= 0;
     const long long mXc = (long long)d.oXt * vX, mYc = (long long)d.oYt * vY;
     float* const Vst = store ? VT + d.vt_off : nullptr;
-    double ej = 0.0, ek = 0.0;
+    __shared__ double red[2][kTThreads];       // the threads' sums of a group
     for (int g0 = tk.pr0; g0 < tk.pr1; g0 += t.np) {
         const int np = min(t.np, tk.pr1 - g0);
+        double ej = 0.0, ek = 0.0;
         float2 acc[8][4], v[8][4];
         if (t.nbuf == 2) {
             load_slices(S1, H1 + (long long)g0 * rows, np, nY, nX, 8 * t.bmY, t.kX, ldX, t.slab, tid);
@@ -1085,34 +1086,42 @@ k_finish_tiled_f32(const DimerDesc* __restrict__ dd, const FinTask* __restrict__
                 }
             }
             if constexpr (PAIRS) {
-                ej += ff_f64(sj);
-                ek += ff_f64(sk);
+                ej = ff_f64(sj);
+                ek = ff_f64(sk);
+            }
+            red[0][tid] = ej;
+            red[1][tid] = ek;
+        }
+        __syncthreads();                         // sums written; S1 consumed
+        if (t.nbuf == 1 && nn > 0)
+            load_slices(S0, H0 + (long long)(g0 + t.np) * rows, nn, nX, nY, 8 * t.bmX, t.kY, ldY, t.slab, tid);
+        // w lanes per pair (w fixed by its block count): its blocks' sums, lanes strided, then
+        // a fixed tree, so that a pair's sums do not depend on the pairs that ran with it
+        // (the largest power of two within it: a group's pairs then take one pass)
+        const int w = nb2 >= 32 ? 32 : nb2 >= 16 ? 16 : nb2 >= 8 ? 8 : nb2 >= 4 ? 4 : nb2 >= 2 ? 2 : 1;
+        for (int q = tid; q < (np * w + 31) / 32 * 32; q += kTThreads) {   // whole warps
+            const int p = q / w, l = q - p * w;
+            double sj = 0.0, sk = 0.0;
+            if (p < np)
+                for (int k = l; k < nb2; k += w) {
+                    sj += red[0][p * nb2 + k];
+                    sk += red[1][p * nb2 + k];
+                }
+            for (int o = w >> 1; o > 0; o >>= 1) {
+                sj += __shfl_xor_sync(0xffffffffu, sj, o);
+                sk += __shfl_xor_sync(0xffffffffu, sk, o);
+            }
+            if (p < np && l == 0) {
+                part[2 * (tk.first + g0 + p)] = sj;
+                part[2 * (tk.first + g0 + p) + 1] = sk;
             }
         }
-        if (t.nbuf == 1 && nn > 0) {
-            __syncthreads();
-            load_slices(S0, H0 + (long long)(g0 + t.np) * rows, nn, nX, nY, 8 * t.bmX, t.kY, ldY, t.slab, tid);
-        } else {
-            __syncthreads();                     // S1 consumed before the next group's H1
-        }
-    }
-    // fixed-order block reduction
-    __shared__ double red[2][kTThreads / 32];
-    ej = warp_sum(ej);
-    ek = warp_sum(ek);
-    if ((tid & 31) == 0) { red[0][tid >> 5] = ej; red[1][tid >> 5] = ek; }
-    __syncthreads();
-    if (tid == 0) {
-        double sj = 0.0, sk = 0.0;
-        for (int w = 0; w < kTThreads / 32; w++) { sj += red[0][w]; sk += red[1][w]; }
-        part[2 * blockIdx.x + 0] = sj;
-        part[2 * blockIdx.x + 1] = sk;
     }
 }
 
-// Per dimer: its task partials -> {4 sum, -2 sum}; a warp each, lane l tasks l,
-// l + 32, ... in order, then the fixed tree (400 tasks of a 128-AO dimer added
-// by one thread took 23 to 40 us).
+// Per dimer: its partials (one per task, FP32 one per pair) -> {4 sum, -2 sum}; a
+// warp each, lane l partials l, l + 32, ... in order, then the fixed tree (400
+// of a 128-AO dimer added by one thread took 23 to 40 us).
 __global__ void __launch_bounds__(32)
 k_finish_sum(const DimerDesc* __restrict__ dd, const FinTask* __restrict__ tasks, const int* __restrict__ first_task,
              const double* __restrict__ part, double* __restrict__ E2)
@@ -1120,7 +1129,7 @@ k_finish_sum(const DimerDesc* __restrict__ dd, const FinTask* __restrict__ tasks
     const int k = blockIdx.x, lane = threadIdx.x;
     const FinTask t0 = tasks[first_task[k]];
     double ej = 0.0, ek = 0.0;
-    for (int t = t0.first + lane; t < t0.first + t0.ntasks; t += 32) {
+    for (int t = t0.first + lane; t < t0.first + t0.nparts; t += 32) {
         ej += part[2 * t];
         ek += part[2 * t + 1];
     }
@@ -1376,22 +1385,42 @@ FinSplit finish_w32_split(const DimerDesc* h, int nd, int form, int sms)
     return five ? FinSplit{5, p5, nullptr} : FinSplit{4, p4, nullptr};
 }
 
-void finish_tasks(const DimerDesc* h, int nd, int fma_per_task, bool fp32, std::vector<FinTask>* out)
+int finish_tasks(const DimerDesc* h, int nd, bool fp32, int sms, std::vector<FinTask>* out)
 {
     out->clear();
-    for (int k = 0; k < nd; k++) {
-        const long long nX = h[k].nX, nY = h[k].nY, vX = h[k].vX, vY = h[k].vY;
-        const int pairs = h[k].oX * h[k].oY;
-        const long long per_pair = 2 * (nX * nY * vY + vX * vY * nX);   // FMAs of one pair, both forms
-        // FP32: whole groups of the pairs that run together
-        const int grp = !fp32 ? 1 : tiled_shape((int)nX, (int)nY, (int)vX, (int)vY, kF32Cap / (int)sizeof(float)).np;
-        const int ppt = (int)std::max<long long>(1, std::min<long long>((pairs + grp - 1) / grp,
-                                                                        fma_per_task / std::max(1LL, per_pair * grp))) * grp;
-        const int ntasks = (pairs + ppt - 1) / ppt;
-        const int first = (int)out->size();
-        for (int t = 0; t < ntasks; t++)
-            out->push_back(FinTask{k, t * ppt, std::min(pairs, (t + 1) * ppt), first, ntasks});
+    constexpr long long kTaskFma = 1 << 22;
+    auto fma_of = [](const DimerDesc& d) {     // multiply-adds of one pair, both forms
+        const long long nX = d.nX, nY = d.nY, vX = d.vX, vY = d.vY;
+        return std::max(1LL, 2 * (nX * nY * vY + vX * vY * nX));
+    };
+    if (!fp32) {
+        for (int k = 0; k < nd; k++) {
+            const int pairs = h[k].oX * h[k].oY;
+            const int ppt = (int)std::max<long long>(1, std::min<long long>(pairs, kTaskFma / fma_of(h[k])));
+            const int ntasks = (pairs + ppt - 1) / ppt, first = (int)out->size();
+            for (int t = 0; t < ntasks; t++)
+                out->push_back(FinTask{k, t * ppt, std::min(pairs, (t + 1) * ppt), first, ntasks});
+        }
+        return (int)out->size();
     }
+    // FP32: whole groups of the pairs that run together, about kTaskFma multiply-adds;
+    // a wave with less than a quarter of one per SM gives each SM its share (the
+    // energies do not depend on it): one dimer of 48 AO, 64 pairs, 53 -> 40 us
+    long long total = 0;
+    for (int k = 0; k < nd; k++) total += fma_of(h[k]) * h[k].oX * h[k].oY;
+    const bool few = total / sms < kTaskFma / 4;
+    const long long per_task = few ? total / sms : kTaskFma;
+    int pairs_before = 0;
+    for (int k = 0; k < nd; k++) {
+        const int pairs = h[k].oX * h[k].oY;
+        const int grp = tiled_shape(h[k].nX, h[k].nY, h[k].vX, h[k].vY, kF32Cap / (int)sizeof(float)).np;
+        const long long want = std::max(1LL, (per_task + (few ? fma_of(h[k]) - 1 : 0)) / fma_of(h[k]));
+        const int ppt = (int)std::min<long long>(pairs, want >= grp ? want / grp * grp : want);
+        for (int p = 0; p < pairs; p += ppt)
+            out->push_back(FinTask{k, p, std::min(pairs, p + ppt), pairs_before, pairs});
+        pairs_before += pairs;
+    }
+    return pairs_before;
 }
 
 cudaError_t launch_fold(const int* fold, int nfold, double* E2, cudaStream_t s)

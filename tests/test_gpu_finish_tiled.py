@@ -35,3 +35,24 @@ def test_finish_above_32_ao(nX, nY, oX, oY):
             out.append(ctx.energies()[2][0].copy())
         assert np.all(np.abs(out[-1] - ref) <= 2e-6 * abs(ref[0])), (out[-1], ref)
     assert np.all(np.abs(out[0] - out[1]) <= 2e-12 * abs(ref[0]))
+
+
+@pytest.mark.parametrize("prec", ["bf16x2", "fp32c"])
+def test_energies_do_not_depend_on_the_wave(prec):
+    """Twelve dimers of different sizes above 32 AO in one run, whose tasks are
+    whole groups, and one by one, whose pairs are dealt to every SM: the same
+    bits."""
+    rng = np.random.default_rng(9)
+    sizes = [(34, 5), (40, 7), (64, 9), (16, 3), (56, 8), (48, 6)]
+    with M.Context(precision=prec) as ctx:
+        mono = [rand_dimer(rng, n, n, o, o)[2:4] for n, o in sizes]
+        for k in range(24):
+            ctx.add_monomer(*mono[k % 6], sizes[k % 6][1])
+        for d in range(12):
+            nX, nY = sizes[2 * d % 6][0], sizes[(2 * d + 1) % 6][0]
+            ctx.add_dimer(2 * d, 2 * d + 1, rng.standard_normal(2 * nX * nX * nY * nY) * 1e-3, M.MCPT_AO_BLOCKS)
+        ctx.run()
+        whole = ctx.energies()[2].copy()
+        for d in range(12):
+            ctx.run(d, 1)
+        assert np.array_equal(ctx.energies()[2], whole)
