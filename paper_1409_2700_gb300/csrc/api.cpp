@@ -140,6 +140,12 @@ struct mcpt_ctx {
     size_t capLists = 0;
     bool lists_dirty = true;
     double* dTot = nullptr;
+    double* mir = nullptr;           // the last run's results in mapped host memory (null: copied on request)
+    size_t capMir = 0;
+    int mirN = 0;                    // monomers of that run (the mirror's layout)
+    double* mirDf = nullptr;         // the same for the density-fitted route
+    size_t capMirDf = 0;
+    int mirDfN = 0;
     int* dFlag = nullptr;            // [0] validation flag, [1] device wait status, [2] the reduction's counter
 
     struct Wave {
@@ -256,6 +262,37 @@ mcpt_status ensure(mcpt_ctx* h, T** p, size_t* cap, size_t bytes)
     *p = static_cast<T*>(q);
     *cap = bytes;
     return MCPT_OK;
+}
+
+// Grow-only mapped host memory; null where there is none to be had (the
+// results are then copied on request).
+void ensure_mirror(mcpt_ctx* h, double** p, size_t* cap, size_t bytes)
+{
+    if (*p && *cap >= bytes) return;
+    if (*p) cudaFreeHost(*p);
+    *p = nullptr;
+    *cap = 0;
+    void* q = nullptr;
+    if (cudaHostAlloc(&q, bytes, cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess) {
+        cudaGetLastError();
+        return;
+    }
+    *p = static_cast<double*>(q);
+    *cap = bytes;
+}
+
+// Results out of a mirror written for n monomers (N now: monomers added since
+// belong to no dimer, their sums are 0) and D dimers.
+void read_mirror(const double* m, size_t n, size_t N, size_t D, double* mon_J, double* mon_K, double* per_dimer,
+                 double* total)
+{
+    for (int f = 0; f < 2; f++)
+        if (double* mon = f ? mon_K : mon_J) {
+            std::memcpy(mon, m + f * n, n * sizeof(double));
+            std::fill(mon + n, mon + N, 0.0);
+        }
+    if (total) std::memcpy(total, m + 2 * n, 2 * sizeof(double));
+    if (per_dimer) std::memcpy(per_dimer, m + 2 * n + 2, 2 * D * sizeof(double));
 }
 
 // The two copy streams of the packed-integral staging buffers and their
@@ -1174,6 +1211,11 @@ static mcpt_status build_plan(mcpt_handle h, mcpt_ctx::Plan& P, int first, int c
     if ((st = ensure_shared(h, &h->dMon, &h->capMon, ((size_t)2 * N + 2 + 4 * kReduceBlocks) * sizeof(double))))
         return st;
     h->dTot = h->dMon + 2 * N;
+    if (!h->mir || h->capMir < mirror_bytes(N, D)) {
+        CK(h, cudaStreamSynchronize(h->stream));   // an earlier run may still write the old one
+        h->epoch++;
+        ensure_mirror(h, &h->mir, &h->capMir, mirror_bytes(N, D));
+    }
     std::vector<size_t> work_off;
     if (is_tensor_form(prec)) {
         size_t total = 0;
@@ -1431,7 +1473,8 @@ static mcpt_status enqueue_run(mcpt_handle h, const mcpt_ctx::Plan& P, const std
         launches++;
     }
     MonomerLists L{h->dLists, h->dLists + N + 1, N};
-    CK(h, launch_reduce(h->dE2, D, L, h->dMon, h->dTot, h->dTot + 2, reduce_counter(h), h->stream));
+    CK(h, launch_reduce(h->dE2, D, L, h->dMon, h->dTot, h->dTot + 2, reduce_counter(h), ResultMirror{h->mir, h->dFlag + 1},
+                        h->stream));
     if (P.coupling) {
         const char* tab = static_cast<const char*>(h->dCoup);
         const CoupTile* tiles = reinterpret_cast<const CoupTile*>(tab + P.off_tiles);
@@ -1550,6 +1593,7 @@ static mcpt_status run_impl(mcpt_handle h, int first, int count)
     }
 
     for (int k = 0; k < count; k++) h->dims[first + k].computed = true;
+    h->mirN = (int)h->mons.size();
     re.runs++;
     re.launches += launches;
     h->stats.waves = (int)W;
@@ -1588,11 +1632,18 @@ mcpt_status mcpt_energies(mcpt_handle h, double* mon_J, double* mon_K, double* p
             return fail(h, MCPT_ESTATE, "mcpt_energies: dimer %zu has not been computed since it was added", d);
     CK(h, cudaSetDevice(h->device));
     CK(h, cudaStreamSynchronize(h->stream));
+    const int N = (int)h->mons.size(), D = (int)h->dims.size();
     int status = 0;
-    CK(h, cudaMemcpy(&status, h->dFlag + 1, sizeof(int), cudaMemcpyDeviceToHost));
+    const double* m = h->mir;
+    const size_t n = h->mirN;
+    if (m) std::memcpy(&status, m + 2 * n + 2 + 2 * (size_t)D, sizeof(int));
+    else CK(h, cudaMemcpy(&status, h->dFlag + 1, sizeof(int), cudaMemcpyDeviceToHost));
     if (status)
         return fail(h, MCPT_ETIMEOUT, "mcpt_energies: a device-side wait gave up (status 0x%x)", status);
-    const int N = (int)h->mons.size(), D = (int)h->dims.size();
+    if (m) {
+        read_mirror(m, n, N, D, mon_J, mon_K, per_dimer, total);
+        return MCPT_OK;
+    }
     if (mon_J) CK(h, cudaMemcpy(mon_J, h->dMon, N * sizeof(double), cudaMemcpyDeviceToHost));
     if (mon_K) CK(h, cudaMemcpy(mon_K, h->dMon + N, N * sizeof(double), cudaMemcpyDeviceToHost));
     if (per_dimer) CK(h, cudaMemcpy(per_dimer, h->dE2, 2 * (size_t)D * sizeof(double), cudaMemcpyDeviceToHost));
@@ -1758,6 +1809,7 @@ mcpt_status mcpt_run_df(mcpt_handle h)
                      (2 * (size_t)D + 2 * (size_t)N + 2 + 4 * kReduceBlocks) * sizeof(double))))
         return st;
     if ((st = ensure(h, &h->dDfLists, &h->capDfLists, lists.size() * sizeof(int)))) return st;
+    ensure_mirror(h, &h->mirDf, &h->capMirDf, mirror_bytes(N, D));   // runs of this route have ended on return
     char* base = static_cast<char*>(h->dDf);
     CK(h, cudaMemcpyAsync(base, dims.data(), (size_t)D * sizeof(DfDim), cudaMemcpyHostToDevice, h->stream));
     CK(h, cudaMemcpyAsync(h->dDfLists, lists.data(), lists.size() * sizeof(int), cudaMemcpyHostToDevice, h->stream));
@@ -1766,9 +1818,11 @@ mcpt_status mcpt_run_df(mcpt_handle h)
                     reinterpret_cast<double*>(base + tab + halfb), E2, h->sms, h->stream));
     MonomerLists L{h->dDfLists, h->dDfLists + N + 1, N};
     CK(h, launch_reduce(E2, D, L, E2 + 2 * (size_t)D, E2 + 2 * (size_t)D + 2 * (size_t)N,
-                        E2 + 2 * (size_t)D + 2 * (size_t)N + 2, reduce_counter(h), h->stream));
+                        E2 + 2 * (size_t)D + 2 * (size_t)N + 2, reduce_counter(h), ResultMirror{h->mirDf, nullptr},
+                        h->stream));
     CK(h, cudaStreamSynchronize(h->stream));   // the host tables go out of scope
     h->df_ran = true;
+    h->mirDfN = N;
     return MCPT_OK;
 }
 
@@ -1779,6 +1833,10 @@ mcpt_status mcpt_df_energies(mcpt_handle h, double* mon_J, double* mon_K, double
     const int N = (int)h->mons.size(), D = (int)h->dfs.size();
     CK(h, cudaSetDevice(h->device));
     CK(h, cudaStreamSynchronize(h->stream));
+    if (h->mirDf) {
+        read_mirror(h->mirDf, h->mirDfN, N, D, mon_J, mon_K, per_dimer, total);
+        return MCPT_OK;
+    }
     const double* E2 = h->dDfOut;
     if (mon_J) CK(h, cudaMemcpy(mon_J, E2 + 2 * (size_t)D, N * sizeof(double), cudaMemcpyDeviceToHost));
     if (mon_K) CK(h, cudaMemcpy(mon_K, E2 + 2 * (size_t)D + N, N * sizeof(double), cudaMemcpyDeviceToHost));
@@ -2118,6 +2176,8 @@ void mcpt_destroy(mcpt_handle h)
     }
     cudaFree(h->dE2);
     cudaFree(h->dMon);
+    cudaFreeHost(h->mir);
+    cudaFreeHost(h->mirDf);
     cudaFree(h->dLists);
     cudaFree(h->dFlag);
     for (cudaEvent_t e : h->rev.pool) cudaEventDestroy(e);

@@ -271,12 +271,21 @@ cudaError_t launch_df(bool fp64, const DfDim* dims, int nd, const DfMax& m, cons
 // each (dimer, first, n) triple of `fold` (device, 3 ints each).
 cudaError_t launch_fold(const int* fold, int nfold, double* E2, cudaStream_t s);
 
+// A copy of the results in mapped host memory (out null: none): per-monomer J
+// then K (2 N), the totals (2), E2 (2 nd), then the device wait status (an int;
+// `status` null: 0).
+struct ResultMirror {
+    double* out;
+    const int* status;
+};
+inline size_t mirror_bytes(int n_mon, int nd) { return (2 * (size_t)n_mon + 2 + 2 * (size_t)nd + 1) * sizeof(double); }
 // Per-monomer halves and the compensated lattice total in one launch.
-// scratch: 4 * kReduceBlocks doubles; cnt: an arrival counter, zero (and left zero).
+// E2 16-byte aligned; scratch: 4 * kReduceBlocks doubles; cnt: an arrival
+// counter, zero (and left zero).
 constexpr int kReduceBlocks = 128;
 cudaError_t launch_reduce(const double* E2, int nd, MonomerLists lists,
                           double* mon /* 2*n_mon */, double* total /* 2 */, double* scratch, unsigned* cnt,
-                          cudaStream_t s);
+                          ResultMirror mir, cudaStream_t s);
 
 // Finiteness check of n doubles; sets *flag to 1 if any is NaN/Inf.
 // Symmetry-packed dimer integrals (MCPT_AO_PACKED): packed_elems(nX, nY)

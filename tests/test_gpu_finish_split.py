@@ -62,3 +62,33 @@ def test_energies_do_not_depend_on_the_split(prec):
         s = 1.0 + d / ND
         ref = oracle.dimer(A * s, K * s, CX, eX, CY, eY, oX, oY)
         assert np.all(np.abs(whole[d] - ref) <= TOL[prec] * abs(ref[0])), (d, whole[d], ref)
+
+
+def test_results_after_monomers_are_added():
+    """The results of a run stay those of the run when monomers are added after
+    it (they belong to no dimer: zero sums), and follow the next run, also of a
+    part, with more dimers and on a replayed graph."""
+    rng = np.random.default_rng(4)
+    A, K, CX, eX, CY, eY = rand_dimer(rng, 10, 12, 2, 3)
+    blocks = np.concatenate([A.ravel(), K.ravel()])
+    with M.Context(precision="fp64") as ctx:
+        ctx.add_monomer(CX, eX, 2)
+        ctx.add_monomer(CY, eY, 3)
+        ctx.add_dimer(0, 1, blocks, M.MCPT_AO_BLOCKS)
+        ctx.run()
+        mj, mk, pd, tot = ctx.energies()
+        for k in range(5):
+            ctx.add_monomer(CX, eX, 2)
+        mj2, mk2, pd2, tot2 = ctx.energies()
+        assert np.array_equal(pd2, pd) and np.array_equal(tot2, tot)
+        assert np.array_equal(mj2[:2], mj) and np.array_equal(mk2[:2], mk)
+        assert not mj2[2:].any() and not mk2[2:].any()
+        for k in range(4):
+            ctx.add_dimer(1, 2 + k, np.concatenate([rand_dimer(rng, 12, 10, 3, 2)[q].ravel() for q in (0, 1)]),
+                          M.MCPT_AO_BLOCKS)
+        for _ in range(3):
+            ctx.run(1, 4)
+            mj3, mk3, pd3, tot3 = ctx.energies()
+            assert np.array_equal(pd3[0], pd[0]) and pd3.shape == (5, 2) and np.all(pd3[1:, 0] < 0)
+            assert abs(tot3[0] - math.fsum(pd3[:, 0])) <= 2.0 ** -51 * np.abs(pd3[:, 0]).sum()
+            assert mj3[6] == 0.0 and abs(mj3[1] - 0.5 * pd3[:, 0].sum()) <= 1e-15 * abs(pd3[:, 0].sum()) * 4
