@@ -1427,7 +1427,7 @@ int finish_tasks(const DimerDesc* h, int nd, bool fp32, int sms, std::vector<Fin
         const int pairs = h[k].oX * h[k].oY;
         const int grp = tiled_shape(h[k].nX, h[k].nY, h[k].vX, h[k].vY, kF32Cap / (int)sizeof(float)).np;
         const long long want = std::max(1LL, (per_task + (few ? fma_of(h[k]) - 1 : 0)) / fma_of(h[k]));
-        const int ppt = (int)std::min<long long>(pairs, want >= grp ? want / grp * grp : want);
+        const int ppt = (int)std::min<long long>(pairs, want >= grp ? want / grp * grp : few ? want : grp);
         for (int p = 0; p < pairs; p += ppt)
             out->push_back(FinTask{k, p, std::min(pairs, p + ppt), pairs_before, pairs});
         pairs_before += pairs;
