@@ -142,7 +142,7 @@ struct mcpt_ctx {
     double* dTot = nullptr;
     double* mir = nullptr;           // the last run's results in mapped host memory (null: copied on request)
     size_t capMir = 0;
-    int mirN = 0;                    // monomers of that run (the mirror's layout)
+    int mirN = 0, mirD = 0;          // monomers and dimers of that run (the mirror's layout)
     double* mirDf = nullptr;         // the same for the density-fitted route
     size_t capMirDf = 0;
     int mirDfN = 0;
@@ -293,6 +293,14 @@ void read_mirror(const double* m, size_t n, size_t N, size_t D, double* mon_J, d
         }
     if (total) std::memcpy(total, m + 2 * n, 2 * sizeof(double));
     if (per_dimer) std::memcpy(per_dimer, m + 2 * n + 2, 2 * D * sizeof(double));
+}
+
+// The last run's device wait status, once the stream has been waited for.
+mcpt_status wait_status(mcpt_ctx* h, int* status)
+{
+    if (h->mir) std::memcpy(status, h->mir + 2 * (size_t)h->mirN + 2 + 2 * (size_t)h->mirD, sizeof(int));
+    else CK(h, cudaMemcpy(status, h->dFlag + 1, sizeof(int), cudaMemcpyDeviceToHost));
+    return MCPT_OK;
 }
 
 // The two copy streams of the packed-integral staging buffers and their
@@ -1264,6 +1272,17 @@ static mcpt_status build_plan(mcpt_handle h, mcpt_ctx::Plan& P, int first, int c
             order[m] = m;
         }
         std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return rows[a] > rows[b]; });
+        auto tiles_of = [&](int m) {
+            const int nt = (mdim[m] + kEdge[cls[m]] - 1) / kEdge[cls[m]];
+            return (long long)nt * (nt + 1) / 2;
+        };
+        // a CTA walks all of its monomer's dimers, so few tiles leave the chip to a
+        // few long chains: below three per SM, the smallest edge throughout (27
+        // monomers of o v = 135, 158 dimers, FP32: 162 tiles 360 us, 405 tiles 254 us)
+        long long ntiles = 0;
+        for (int m = 0; m < N; m++) ntiles += tiles_of(m);
+        if (ntiles < 3LL * h->sms)
+            for (int m = 0; m < N; m++) cls[m] = 2;
         std::vector<CoupTile> tiles;
         for (int c = 0; c < 3; c++) {
             const size_t before = tiles.size();
@@ -1594,6 +1613,7 @@ static mcpt_status run_impl(mcpt_handle h, int first, int count)
 
     for (int k = 0; k < count; k++) h->dims[first + k].computed = true;
     h->mirN = (int)h->mons.size();
+    h->mirD = (int)h->dims.size();
     re.runs++;
     re.launches += launches;
     h->stats.waves = (int)W;
@@ -1634,14 +1654,11 @@ mcpt_status mcpt_energies(mcpt_handle h, double* mon_J, double* mon_K, double* p
     CK(h, cudaStreamSynchronize(h->stream));
     const int N = (int)h->mons.size(), D = (int)h->dims.size();
     int status = 0;
-    const double* m = h->mir;
-    const size_t n = h->mirN;
-    if (m) std::memcpy(&status, m + 2 * n + 2 + 2 * (size_t)D, sizeof(int));
-    else CK(h, cudaMemcpy(&status, h->dFlag + 1, sizeof(int), cudaMemcpyDeviceToHost));
+    if (mcpt_status st = wait_status(h, &status)) return st;
     if (status)
         return fail(h, MCPT_ETIMEOUT, "mcpt_energies: a device-side wait gave up (status 0x%x)", status);
-    if (m) {
-        read_mirror(m, n, N, D, mon_J, mon_K, per_dimer, total);
+    if (h->mir) {
+        read_mirror(h->mir, h->mirN, N, D, mon_J, mon_K, per_dimer, total);
         return MCPT_OK;
     }
     if (mon_J) CK(h, cudaMemcpy(mon_J, h->dMon, N * sizeof(double), cudaMemcpyDeviceToHost));
@@ -1664,7 +1681,7 @@ mcpt_status mcpt_coupling(mcpt_handle h, int X, double* R)
     const size_t mm = (size_t)h->mons[X].nocc * (h->mons[X].nao - h->mons[X].nocc);
     CK(h, cudaStreamSynchronize(h->stream));
     int status = 0;
-    CK(h, cudaMemcpy(&status, h->dFlag + 1, sizeof(int), cudaMemcpyDeviceToHost));
+    if (mcpt_status es = wait_status(h, &status)) return es;
     if (status) return fail(h, MCPT_ETIMEOUT, "mcpt_coupling: a device-side wait gave up (status 0x%x)", status);
     CK(h, cudaMemcpy(R, h->dR + h->r_off[X], mm * mm * sizeof(double), cudaMemcpyDeviceToHost));
     return MCPT_OK;
@@ -1704,7 +1721,7 @@ mcpt_status mcpt_singles(mcpt_handle h, const double* t, double* s)
     CK(h, cudaMemcpyAsync(s, h->dS1 + M, M * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
     CK(h, cudaStreamSynchronize(h->stream));
     int status = 0;
-    CK(h, cudaMemcpy(&status, h->dFlag + 1, sizeof(int), cudaMemcpyDeviceToHost));
+    if (mcpt_status es = wait_status(h, &status)) return es;
     if (status) return fail(h, MCPT_ETIMEOUT, "mcpt_singles: a device-side wait gave up (status 0x%x)", status);
     return MCPT_OK;
 }
