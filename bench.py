@@ -324,7 +324,7 @@ def our_arm(args, ws, rank, local):
         traffic = tpd * w.n_dimers / st.waves if (tpd and uniform) else None
         roof = {"bound": "hbm", "achieved": achieved, "peak": peaks["hbm_gbs"], "unit": "GB/s",
                 "frac": achieved / peaks["hbm_gbs"], "traffic": traffic,
-                "kernel": "k_half_tc_rank" if args.precision in ("tf32", "bf16x3", "bf16x2", "fp64e") else "k_half_fp32c",
+                "kernel": "k_half_tc_rank" if args.precision in ("tf32", "bf16x3", "bf16x2", "fp64e") else "k_half_fp32c_tiles",
                 "peak_kind": peak_kind}
 
     line = {
@@ -830,7 +830,7 @@ def streamed_arm(args, ws, rank, local):
         roof = {"bound": "hbm", "achieved": achieved, "peak": peaks["hbm_gbs"], "unit": "GB/s",
                 "frac": achieved / peaks["hbm_gbs"],
                 "traffic": tpd * timed_dimers / nsteps if (tpd and uniform) else None,
-                "kernel": "k_half_tc_rank" if args.precision in ("tf32", "bf16x3", "bf16x2", "fp64e") else "k_half_fp32c",
+                "kernel": "k_half_tc_rank" if args.precision in ("tf32", "bf16x3", "bf16x2", "fp64e") else "k_half_fp32c_tiles",
                 "peak_kind": peak_kind,
                 "per": "one wave's first-half launch (traffic scaled from the ncu capture per dimer)"}
     line = {

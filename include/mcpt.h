@@ -109,7 +109,9 @@ typedef struct {
     void *stream;             /* cudaStream_t to run on, or NULL for a library-owned stream */
     mcpt_precision precision; /* see above */
     int validate;             /* 1: reject non-finite C / eps / integrals (adds a pass over inputs) */
-    size_t wave_bytes;        /* cap on per-run device scratch; dimers run in waves under it (0 = 1 GiB) */
+    size_t wave_bytes;        /* cap on per-run device scratch; dimers run in waves under it (0 = 1 GiB).
+                                 MCPT_FP32C takes up to a quarter of it for its first half's slots when that
+                                 holds one per SM (and no mem_cap_bytes is set) */
     const char *tune_cache;   /* path of the autotuner's cache, or NULL: with a path, each tensor-core
                                  wave's launch choices (kernel variant, staging depth, grid) are timed on
                                  the first plan of its shape signature and kept in that text file */
@@ -204,7 +206,9 @@ mcpt_status mcpt_update_dimer(mcpt_handle h, int id, const double *ao_eri, mcpt_
  * the same flags and ownership rules.  For MCPT_AO_PACKED the dimers whose
  * data lie back to back in the buffer are copied together, in chunks of up
  * to 256 MB and 64 dimers through two device staging buffers (one copy
- * stream each), and each chunk is expanded by one launch: with pinned memory and MCPT_UPDATE_ASYNC the
+ * stream each), and each chunk is expanded by one launch; with validate = 1 the
+ * data is checked by several host threads beside the first copies, before
+ * anything is expanded: with pinned memory and MCPT_UPDATE_ASYNC the
  * copies run at the link's bandwidth instead of being paced by one call per
  * dimer.  A dimer whose integrals were borrowed device memory gets storage
  * of its own (its run plan is rebuilt).  Not a step of the paper's method: the
