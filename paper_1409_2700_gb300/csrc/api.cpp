@@ -264,19 +264,22 @@ mcpt_status ensure(mcpt_ctx* h, T** p, size_t* cap, size_t bytes)
     return MCPT_OK;
 }
 
-// Grow-only mapped host memory; null where there is none to be had (the
-// results are then copied on request).
+// Grow-only mapped host memory that keeps its contents (a run that then fails
+// leaves the last run's results readable); zeros at first, null where there is
+// none to be had (the results are then copied on request).
 void ensure_mirror(mcpt_ctx* h, double** p, size_t* cap, size_t bytes)
 {
     if (*p && *cap >= bytes) return;
-    if (*p) cudaFreeHost(*p);
-    *p = nullptr;
-    *cap = 0;
     void* q = nullptr;
     if (cudaHostAlloc(&q, bytes, cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess) {
         cudaGetLastError();
-        return;
+        q = nullptr;
+        bytes = 0;
+    } else {
+        std::memset(q, 0, bytes);
+        if (*p) std::memcpy(q, *p, *cap);
     }
+    if (*p) cudaFreeHost(*p);
     *p = static_cast<double*>(q);
     *cap = bytes;
 }
@@ -1219,11 +1222,6 @@ static mcpt_status build_plan(mcpt_handle h, mcpt_ctx::Plan& P, int first, int c
     if ((st = ensure_shared(h, &h->dMon, &h->capMon, ((size_t)2 * N + 2 + 4 * kReduceBlocks) * sizeof(double))))
         return st;
     h->dTot = h->dMon + 2 * N;
-    if (!h->mir || h->capMir < mirror_bytes(N, D)) {
-        CK(h, cudaStreamSynchronize(h->stream));   // an earlier run may still write the old one
-        h->epoch++;
-        ensure_mirror(h, &h->mir, &h->capMir, mirror_bytes(N, D));
-    }
     std::vector<size_t> work_off;
     if (is_tensor_form(prec)) {
         size_t total = 0;
@@ -1424,7 +1422,10 @@ static mcpt_status build_plan(mcpt_handle h, mcpt_ctx::Plan& P, int first, int c
         }
         P.waves.push_back(wv);
     }
-    CK(h, cudaStreamSynchronize(h->stream));
+    CK(h, cudaStreamSynchronize(h->stream));   // an earlier run may still write the mirror
+    const double* mir = h->mir;
+    ensure_mirror(h, &h->mir, &h->capMir, mirror_bytes(N, D));   // last: nothing of the plan can fail after it
+    if (h->mir != mir) h->epoch++;
     P.prec = prec;
     P.first = first;
     P.count = count;
