@@ -13,7 +13,6 @@
 // CTAs' partial energies are added per dimer in fixed order (k_df_sum).
 #include "internal.h"
 #include "convert.h"
-#include "ff.h"
 
 #include <algorithm>
 
@@ -218,13 +217,32 @@ k_df_half(const DfDim* __restrict__ dims, const double* __restrict__ C, float* _
 constexpr int kDQ = 16;                        // Q values per staged chunk
 constexpr int kDJ = 5;                         // most j of a CTA
 
-// One energy term: v^2 and v w as exact products on FP32 pairs, times D = 1/x
-// and summed on pairs too (~2^-45, ff.h).
-__device__ __forceinline__ void df_term(FF& sj, FF& sk, float v, float w, FF D)
+// FP64 from FP32, exact for every value: normal ones on the integer pipes, the
+// rest (zeros, subnormals, infinities, NaN) by the conversion unit, out of line
+// so that it does not issue for the others.
+__device__ __noinline__ double convert(float f) { return (double)f; }
+
+__device__ __forceinline__ double widen(float f)
 {
-    const float jh = __fmul_rn(v, v), kh = __fmul_rn(v, w);
-    ff_mac(sj, FF{jh, fmaf(v, v, -jh)}, D);
-    ff_mac(sk, FF{kh, fmaf(v, w, -kh)}, D);
+    const unsigned e = (__float_as_uint(f) >> 23) & 0xFFu;
+    return e - 1u < 254u ? f64_from_f32(f) : convert(f);
+}
+
+__device__ __noinline__ double divide(double v, double x) { return v / x; }
+
+// One energy term in FP64, v and w the unscaled (ia|jb) and (ib|ja), x the
+// denominator: v / x to FP64 rounding by two Newton steps (convert.h) where |x|
+// lies in 2^+-124, as the differences of orbital energies do, else by division.
+// On FP32 pairs (2^-45) with the squares formed in FP32 the terms were less
+// accurate and overflowed where s v does not.  (Out of line the rare paths cost
+// no registers of the loop above.)
+__device__ __forceinline__ void df_term(double& sj, double& sk, float v, float w, double x)
+{
+    const double vd = widen(v);
+    const unsigned e = ((unsigned)__double2hiint(x) >> 20) & 0x7FFu;
+    const double t = e - 899u < 249u ? div_newton<2>(vd, x) : divide(vd, x);
+    sj = fma(t, vd, sj);
+    sk = fma(t, widen(w), sk);
 }
 
 // The j block [j0, j0 + JB) of occupied i: a thread holds 4 a x 4 b x JB values of
@@ -310,26 +328,24 @@ __device__ __forceinline__ void df_pairs(const DfDim& d, const double* __restric
             __syncthreads();                   // chunk consumed before its buffer is refilled
         }
         if (t0 + tid >= nt) continue;
-        FF sj{0.f, 0.f}, sk{0.f, 0.f}, eb[4];
+        double eb[4];
 #pragma unroll
-        for (int y = 0; y < 4; y++) eb[y] = ff_split(b0 + y < vY ? eps[d.eY + oY + b0 + y] : 0.0);
+        for (int y = 0; y < 4; y++) eb[y] = b0 + y < vY ? eps[d.eY + oY + b0 + y] : 0.0;
 #pragma unroll
         for (int x = 0; x < 4; x++) {
             if (a0 + x >= vX) break;
             const double ea = eps[d.eX + oX + a0 + x];
 #pragma unroll
             for (int j = 0; j < JB; j++) {
-                const FF eija = ff_split(ei + eps[d.eY + j0 + j] - ea);
+                const double eija = ei + eps[d.eY + j0 + j] - ea;
 #pragma unroll
                 for (int y = 0; y < 4; y++) {
                     if (b0 + y >= vY) break;
-                    df_term(sj, sk, y & 1 ? v[j][x][y / 2].y : v[j][x][y / 2].x,
-                            x & 1 ? w[j][y][x / 2].y : w[j][y][x / 2].x, ff_rcp(ff_sub(eija, eb[y])));
+                    df_term(ej, ek, y & 1 ? v[j][x][y / 2].y : v[j][x][y / 2].x,
+                            x & 1 ? w[j][y][x / 2].y : w[j][y][x / 2].x, eija - eb[y]);
                 }
             }
         }
-        ej += ff_f64(sj);
-        ek += ff_f64(sk);
     }
 }
 
@@ -366,9 +382,9 @@ k_df_pair(const DfDim* __restrict__ dims, const double* __restrict__ eps, const 
     if (threadIdx.x == 0) {
         double sj = 0.0, sk = 0.0;
         for (int w = 0; w < (int)(blockDim.x >> 5); w++) { sj += red[0][w]; sk += red[1][w]; }
-        const double s2 = d.s * d.s;
-        part[2 * (d.p_off + k)] = 4.0 * s2 * sj;
-        part[2 * (d.p_off + k) + 1] = -2.0 * s2 * sk;
+        // s and s again: its square alone may leave FP64's range where s v does not
+        part[2 * (d.p_off + k)] = d.s * (d.s * (4.0 * sj));
+        part[2 * (d.p_off + k) + 1] = d.s * (d.s * (-2.0 * sk));
     }
 }
 
