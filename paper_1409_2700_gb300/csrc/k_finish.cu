@@ -1387,12 +1387,22 @@ cudaError_t launch_finish_ff(const DimerDesc* d_desc, int nd, int max_ao, const 
 // 176).  FP32 waves of more than six dimers per SM are bound by the FP32
 // pipes either way, and staging the coefficients once per dimer is then the
 // cheaper: 1036 dimers 256 against 266, 2248 dimers 513 against 557.
+// FP64E (two CTAs per SM, 74 us of pair arithmetic per round of four pairs, 0.18
+// of that to stage the coefficients) takes whichever of the two fills its last
+// set of CTAs better: 25 pairs, one CTA per dimer against seven, 158 dimers 530 /
+// 350, 304 554 / 630, 1036 2129 / 2104, 1216 2153 / 2466, 2216 4230 / 4460; 9
+// pairs against three, 158 187 / 153, 1036 736 / 804; two to five CTAs for 25
+// pairs were slower than the better of these at every size.
 FinSplit finish_w32_split(const DimerDesc* h, int nd, int form, int sms)
 {
     int pairs = 1;
     for (int k = 0; k < nd; k++) pairs = std::max(pairs, h[k].oX * h[k].oY);
     if ((form == FIN_F32_PAIRS || form == FIN_F32_F64EPI) && nd > 6 * sms) return FinSplit{4, 1, nullptr};
     const int p4 = (pairs + 3) / 4, p5 = (pairs + 4) / 5;
+    if (form == FIN_FF) {                      // in hundredths of a round
+        auto sets = [&](long long ctas) { return (ctas + 2 * sms - 1) / (2 * sms); };
+        if (sets(nd) * (100 * p4 + 18) < sets((long long)nd * p4) * 118) return FinSplit{4, 1, nullptr};
+    }
     const bool five = (long long)nd * p5 <= sms && (long long)nd * p4 > sms;
     return five ? FinSplit{5, p5, nullptr} : FinSplit{4, p4, nullptr};
 }
