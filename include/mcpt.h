@@ -214,7 +214,9 @@ mcpt_status mcpt_update_dimer(mcpt_handle h, int id, const double *ao_eri, mcpt_
  * of its own (its run plan is rebuilt).  Not a step of the paper's method: the
  * ingest of a sequence of lattices.
  * Errors: EINVAL (range, NULL, layout, flags, non-finite with validate=1),
- *   ENOMEM, ECUDA. */
+ *   ENOMEM, ECUDA; for MCPT_AO_PACKED EINVAL and ENOMEM leave every dimer and
+ *   the last run's results as they were, and after any error the caller's
+ *   buffer is no longer read. */
 mcpt_status mcpt_update_dimers(mcpt_handle h, int first, int count, const double *ao_eri, const size_t *offsets,
                                mcpt_ao_layout layout, int flags);
 

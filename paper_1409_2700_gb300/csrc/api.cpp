@@ -882,11 +882,16 @@ mcpt_status mcpt_update_dimers(mcpt_handle h, int first, int count, const double
         k += c.n;
     }
     if ((st = ensure_copy_streams(h))) return st;
+    // every allocation before the first change: one that fails leaves the
+    // dimers, their results and the plans as they were
     const int sb0 = h->pack_next;
+    size_t most[2] = {0, 0};
+    for (size_t c = 0; c < chunks.size(); c++)
+        most[(sb0 + c) & 1] = std::max(most[(sb0 + c) & 1], chunks[c].elems * sizeof(double));
+    for (int sb = 0; sb < 2; sb++)
+        if (most[sb] && (st = ensure(h, &h->dPack[sb], &h->capPack[sb], most[sb]))) return st;
     auto copy = [&](size_t c) -> mcpt_status {
         const int sb = (sb0 + (int)c) & 1;
-        mcpt_status e = ensure(h, &h->dPack[sb], &h->capPack[sb], chunks[c].elems * sizeof(double));
-        if (e) return e;
         CK(h, cudaStreamWaitEvent(h->copy_stream[sb], h->ev_free[sb], 0));    // its last expansion has read it
         CK(h, cudaMemcpyAsync(h->dPack[sb], src[chunks[c].k], chunks[c].elems * sizeof(double),
                               cudaMemcpyHostToDevice, h->copy_stream[sb]));
@@ -902,32 +907,37 @@ mcpt_status mcpt_update_dimers(mcpt_handle h, int first, int count, const double
         // the first two chunks go over while the host reads the data; nothing
         // is expanded into the dimers' storage before all of it is found finite
         for (; copied < std::min<size_t>(2, chunks.size()); copied++)
-            if ((st = copy(copied))) break;
-        if (st) return drain(st);
+            if ((st = copy(copied))) return drain(st);
         const int bad = first_non_finite(src.data(), np.data(), count);
         if (bad >= 0)
             return drain(fail(h, MCPT_EINVAL, "mcpt_update_dimers: non-finite integral (dimer %d)", first + bad));
     }
+    auto blk_of = [&](const DimerRec& r) {
+        const size_t nX = h->mons[r.X].nao, nY = h->mons[r.Y].nao;
+        return nX * nX * nY * nY;
+    };
+    for (int k = 0; k < count; k++) {
+        DimerRec& r = h->dims[first + k];
+        if (r.owned) continue;                // else only ever borrowed device data: storage of its own
+        void* dst = nullptr;
+        if ((st = arena_alloc(h, 2 * blk_of(r) * sizeof(double), &dst))) return drain(st);
+        r.owned = static_cast<double*>(dst);
+    }
     for (int k = 0; k < count; k++) {
         DimerRec& r = h->dims[first + k];
         const int nX = h->mons[r.X].nao, nY = h->mons[r.Y].nao;
-        const size_t blk = (size_t)nX * nX * nY * nY;
-        if (!r.owned) {                       // only ever borrowed device data: storage of its own
-            void* dst = nullptr;
-            if ((st = arena_alloc(h, 2 * blk * sizeof(double), &dst))) return drain(st);
-            r.owned = static_cast<double*>(dst);
-        }
         if (r.E[0] != r.owned) {              // the record points at borrowed data: back to the storage
             r.E[0] = r.owned;
             r.st[0][0] = (long long)nX * nY * nY; r.st[0][1] = (long long)nY * nY; r.st[0][2] = nY;
-            r.E[1] = r.owned + blk;
+            r.E[1] = r.owned + blk_of(r);
             r.st[1][0] = (long long)nY * nY * nX; r.st[1][1] = (long long)nY * nX; r.st[1][2] = nX;
             moved = true;
         }
+        r.computed = false;                   // also where a launch fails between the chunks
     }
+    h->coupled = false;
     if (moved) drop_plans(h);                 // the tensor maps name the old addresses
-    for (size_t c = 0; c < chunks.size(); c++) {
-        if (c >= copied && (st = copy(c))) return st;
+    auto expand = [&](size_t c) -> mcpt_status {
         const int sb = h->pack_next, k = chunks[c].k;
         h->pack_next ^= 1;
         CK(h, cudaStreamWaitEvent(h->stream, h->ev_copied[sb], 0));
@@ -941,9 +951,12 @@ mcpt_status mcpt_update_dimers(mcpt_handle h, int first, int count, const double
         }
         CK(h, launch_unpack_batch(B, h->stream));
         CK(h, cudaEventRecord(h->ev_free[sb], h->stream));
+        return MCPT_OK;
+    };
+    for (size_t c = 0; c < chunks.size(); c++) {
+        if (c >= copied && (st = copy(c))) return drain(st);
+        if ((st = expand(c))) return drain(st);
     }
-    for (int k = 0; k < count; k++) h->dims[first + k].computed = false;
-    h->coupled = false;
     if (!(flags & MCPT_UPDATE_ASYNC)) CK(h, cudaStreamSynchronize(h->stream));
     return MCPT_OK;
 }
