@@ -111,7 +111,11 @@ typedef struct {
     int validate;             /* 1: reject non-finite C / eps / integrals (adds a pass over inputs) */
     size_t wave_bytes;        /* cap on per-run device scratch; dimers run in waves under it (0 = 1 GiB).
                                  MCPT_FP32C takes up to a quarter of it for its first half's slots when that
-                                 holds one per SM (and no mem_cap_bytes is set) */
+                                 holds one per SM (and no mem_cap_bytes is set) and the device has the
+                                 memory: they are taken last and given back when memory runs out (but for
+                                 a handle whose run was launched into a caller's stream capture).  Without
+                                 them a slower kernel runs, whose results may differ from the other's in
+                                 the last FP32 bit of the half-transformed integrals */
     const char *tune_cache;   /* path of the autotuner's cache, or NULL: with a path, each tensor-core
                                  wave's launch choices (kernel variant, staging depth, grid) are timed on
                                  the first plan of its shape signature and kept in that text file */

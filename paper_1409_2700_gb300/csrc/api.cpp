@@ -113,8 +113,9 @@ struct mcpt_ctx {
 
     void* dH = nullptr;              // first-half result of one wave (shared by every plan)
     size_t capH = 0;
-    void* dFc = nullptr;             // FP32C: tile counter and per-CTA slots of the first half (shared)
-    size_t capFc = 0;
+    void* dFc = nullptr;             // FP32C: tile counter and per-CTA slots of the first half (shared;
+    size_t capFc = 0;                // given back when memory runs out, unless a caller's graph uses them)
+    bool fc_captured = false;        // a run with slots was launched into a caller's capture
     void* dVT = nullptr;             // coupling: every dimer's (ia|jb) and T = vD
     size_t capVT = 0;
     void* dCoup = nullptr;           // coupling tables: tiles, per-dimer info, monomer sizes, R offsets
@@ -226,26 +227,44 @@ mcpt_status fail(mcpt_ctx* h, mcpt_status st, const char* fmt, ...)
                         #call);                                                                  \
     } while (0)
 
-mcpt_status dev_alloc(mcpt_ctx* h, void** p, size_t bytes)
-{
-    if (h->mem_cap && h->mem_used + bytes > h->mem_cap)
-        return fail(h, MCPT_ENOMEM, "device memory cap of %zu bytes reached (%zu in use, %zu requested)",
-                    h->mem_cap, h->mem_used, bytes);
-    cudaError_t e = cudaMalloc(p, bytes);
-    if (e != cudaSuccess) {
-        cudaGetLastError();
-        return fail(h, MCPT_ENOMEM, "cudaMalloc(%zu) failed: %s", bytes, cudaGetErrorString(e));
-    }
-    h->mem_used += bytes;
-    return MCPT_OK;
-}
-
 void dev_free(mcpt_ctx* h, void* p, size_t bytes)
 {
     if (p) {
         cudaFree(p);
         h->mem_used -= bytes;
     }
+}
+
+// Give the FP32C slots back (they only make a run faster); false if there are
+// none to be had.  The plans that use them are rebuilt.
+bool give_back_slots(mcpt_ctx* h)
+{
+    if (!h->dFc || h->fc_captured) return false;
+    if (h->stream) cudaStreamSynchronize(h->stream);
+    dev_free(h, h->dFc, h->capFc);
+    h->dFc = nullptr;
+    h->capFc = 0;
+    h->epoch++;
+    return true;
+}
+
+// wanted: memory the caller can do without; it takes nothing from the slots.
+mcpt_status dev_alloc(mcpt_ctx* h, void** p, size_t bytes, bool wanted = false)
+{
+    if (h->mem_cap && h->mem_used + bytes > h->mem_cap)
+        return fail(h, MCPT_ENOMEM, "device memory cap of %zu bytes reached (%zu in use, %zu requested)",
+                    h->mem_cap, h->mem_used, bytes);
+    cudaError_t e = cudaMalloc(p, bytes);
+    if (e != cudaSuccess && !wanted && give_back_slots(h)) {
+        cudaGetLastError();
+        e = cudaMalloc(p, bytes);
+    }
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        return fail(h, MCPT_ENOMEM, "cudaMalloc(%zu) failed: %s", bytes, cudaGetErrorString(e));
+    }
+    h->mem_used += bytes;
+    return MCPT_OK;
 }
 
 // Grow-only device buffer.
@@ -358,7 +377,7 @@ mcpt_status arena_alloc(mcpt_ctx* h, size_t bytes, void** out)
     if (bytes > h->arena_left) {
         size_t chunk = std::max(bytes, (size_t)512 << 20);
         void* p = nullptr;
-        mcpt_status st = dev_alloc(h, &p, chunk);
+        mcpt_status st = dev_alloc(h, &p, chunk, chunk > bytes);
         if (st) {
             if (chunk == bytes) return st;
             h->err.clear();
@@ -1123,7 +1142,8 @@ static mcpt_status build_plan(mcpt_handle h, mcpt_ctx::Plan& P, int first, int c
     // FP32C: a quarter of the run's scratch for the first half's slots, one
     // per resident CTA.  With room for fewer than one slot per SM, or with a
     // memory cap (whose every byte may be wanted for integrals added later),
-    // the kernel that needs no slots runs and H has all of the scratch.
+    // the kernel that needs no slots runs and H has all of the scratch.  They
+    // are allocated after everything the plan needs.
     P.fc_slots = 0;
     P.fc_slot_bytes = 0;
     size_t wave_cap = h->wave_bytes;
@@ -1207,11 +1227,6 @@ static mcpt_status build_plan(mcpt_handle h, mcpt_ctx::Plan& P, int first, int c
     if ((st = ensure(h, &P.dDesc, &P.capDesc, ndesc * (sizeof(DimerDesc) + sizeof(unsigned))))) return st;
     unsigned* const fin_cnt = reinterpret_cast<unsigned*>(P.dDesc + ndesc);
     if ((st = ensure_shared(h, &h->dH, &h->capH, max_wave_h))) return st;
-    if (P.fc_slots &&
-        ensure_shared(h, &h->dFc, &h->capFc, kFp32cCounterBytes + P.fc_slots * P.fc_slot_bytes) != MCPT_OK) {
-        h->err.clear();
-        P.fc_slots = 0;                        // no room on the device: the kernel without slots
-    }
     if (!fold.empty() && (st = ensure(h, &P.dFold, &P.capFold, fold.size() * sizeof(int)))) return st;
     // per-dimer results, then the results of split dimers' blocks (kept across
     // plans: a larger array copies the dimers' results over)
@@ -1435,6 +1450,16 @@ static mcpt_status build_plan(mcpt_handle h, mcpt_ctx::Plan& P, int first, int c
         }
         P.waves.push_back(wv);
     }
+    // the slots, if there is room for one per resident CTA or at least per SM:
+    // nothing that a run needs is refused for them (give_back_slots)
+    const int want = std::exchange(P.fc_slots, 0);
+    for (int n : {want, std::min(want, h->sms)}) {
+        if (!n || P.fc_slots) continue;
+        const size_t bytes = kFp32cCounterBytes + n * P.fc_slot_bytes;
+        if (h->dFc && h->capFc < bytes) h->epoch++;      // a smaller one, which other plans name, goes
+        if (ensure(h, &h->dFc, &h->capFc, bytes) == MCPT_OK) P.fc_slots = n;
+        else h->err.clear();
+    }
     CK(h, cudaStreamSynchronize(h->stream));   // an earlier run may still write the mirror
     const double* mir = h->mir;
     ensure_mirror(h, &h->mir, &h->capMir, mirror_bytes(N, D));   // last: nothing of the plan can fail after it
@@ -1624,6 +1649,7 @@ static mcpt_status run_impl(mcpt_handle h, int first, int count)
         mcpt_status st = enqueue_run(h, P, nullptr, &launches);
         if (st) return st;
     }
+    if (cap != cudaStreamCaptureStatusNone && P.fc_slots) h->fc_captured = true;
 
     for (int k = 0; k < count; k++) h->dims[first + k].computed = true;
     h->mirN = (int)h->mons.size();
