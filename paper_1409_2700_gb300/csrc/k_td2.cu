@@ -731,11 +731,15 @@ template <typename TI, typename TO>
 cudaError_t launch_qstep(const QStep<TI, TO>* steps, int nd, int max_m, int max_n, cudaStream_t s)
 {
     if (nd <= 0) return cudaSuccess;
-    const dim3 big((max_m + 127) / 128, (max_n + kQN - 1) / kQN, nd), grid((max_m + 63) / 64, big.y, nd);
-    if (sizeof(TO) == 4 && (long long)big.x * big.y * nd >= 4LL * sm_count())
-        k_qstep<TI, TO, 128><<<big, kQThreads, 0, s>>>(steps);
-    else
-        k_qstep<TI, TO, 64><<<grid, kQThreads, 0, s>>>(steps);
+    if constexpr (sizeof(TO) == 4) {
+        const dim3 big((max_m + 127) / 128, (max_n + kQN - 1) / kQN, nd);
+        if ((long long)big.x * big.y * nd >= 4LL * sm_count()) {
+            k_qstep<TI, TO, 128><<<big, kQThreads, 0, s>>>(steps);
+            return cudaGetLastError();
+        }
+    }
+    const dim3 grid((max_m + 63) / 64, (max_n + kQN - 1) / kQN, nd);
+    k_qstep<TI, TO, 64><<<grid, kQThreads, 0, s>>>(steps);
     return cudaGetLastError();
 }
 
