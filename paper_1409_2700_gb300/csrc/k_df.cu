@@ -203,8 +203,9 @@ k_df_half(const DfDim* __restrict__ dims, const double* __restrict__ C, float* _
 #pragma unroll
                 for (int r = 0; r < kHRows; r++) {
                     if (gr * kHRows + r < rows) {
-                        float* out = o < oX ? (hy ? xy : xx) + ((qb + q) * oX + o) * vq
-                                            : (hy ? yy : yx) + ((qb + q) * oY + o - oX) * vq;
+                        // (naux o v of a factor set above 64 GB passes 32 bits)
+                        float* out = o < oX ? (hy ? xy : xx) + ((long long)(qb + q) * oX + o) * vq
+                                            : (hy ? yy : yx) + ((long long)(qb + q) * oY + o - oX) * vq;
                         out[c] = a2[r].x + a2[r].y;
                     }
                     if (++o == ot) { o = 0; q++; }
