@@ -10,7 +10,8 @@
 // R is symmetric, so only tiles with q0 >= p0 run, each writing R[p][q] and
 // its mirror R[q][p] for p <= q (R is exactly symmetric).  A monomer's tiles
 // have edge 64, 48 or 32, whichever covers its o v rows with the least padded
-// work, one launch per edge.  A CTA walks the monomer's dimers in ascending
+// work, or 32 throughout where those come to fewer than three tiles per SM (few
+// long chains; api.cpp, build_plan), one launch per edge.  A CTA walks the monomer's dimers in ascending
 // order and their rows in chunks of 32 (16 in FP64), staged in shared memory
 // by cp.async into two buffers: the next chunk is in flight while the
 // current one is summed.  (Chunks of 16 or 24 rows, which fit five CTAs of
