@@ -109,6 +109,8 @@ k_df_half(const DfDim* __restrict__ dims, const double* __restrict__ C, float* _
     };
     stage(VX, OX, C + d.cX, nX, oX, nXp, vXq, sX);
     stage(VY, OY, C + d.cY, nY, oY, nYp, vYq, sY);
+    // the four blocks (32-bit indices below count rows of four: naux o v alone
+    // passes 2^31 above 64 GB of factors, a quarter of it not within the device)
     float* xx = half + d.h_off;
     float* yy = xx + (long long)naux * oX * vXq;
     float* xy = yy + (long long)naux * oY * vYq;
@@ -203,10 +205,9 @@ k_df_half(const DfDim* __restrict__ dims, const double* __restrict__ C, float* _
 #pragma unroll
                 for (int r = 0; r < kHRows; r++) {
                     if (gr * kHRows + r < rows) {
-                        // (naux o v of a factor set above 64 GB passes 32 bits)
-                        float* out = o < oX ? (hy ? xy : xx) + ((long long)(qb + q) * oX + o) * vq
-                                            : (hy ? yy : yx) + ((long long)(qb + q) * oY + o - oX) * vq;
-                        out[c] = a2[r].x + a2[r].y;
+                        float4* out = o < oX ? reinterpret_cast<float4*>(hy ? xy : xx) + ((qb + q) * oX + o) * (vq / 4)
+                                             : reinterpret_cast<float4*>(hy ? yy : yx) + ((qb + q) * oY + o - oX) * (vq / 4);
+                        reinterpret_cast<float*>(out)[c] = a2[r].x + a2[r].y;
                     }
                     if (++o == ot) { o = 0; q++; }
                 }
