@@ -324,6 +324,7 @@ enum TcKind { TC_TF32 = 0, TC_BF16X3 = 1, TC_BF16X2 = 2, TC_FP64E = 3 };
 struct TcLaunch {
     const void* items;          // device TcItem array
     int n_items;
+    int split;                  // M-tiles of 128 / split rows
     const void* maps;           // device CUtensorMap array, [dimer][form]
     const DimerDesc* desc;      // device descriptors of the launch's dimers
     const float* Cf;            // FP32 coefficient pool

@@ -46,8 +46,8 @@ namespace mcpt {
 
 struct TcItem {
     int dimer;   // index within the launch's descriptor array
-    int form;    // 0: A block, 1: K block
-    int p1t;     // p1 values per M-tile (tile_p1)
+    short form;  // 0: A block, 1: K block
+    short p1t;   // p1 values per M-tile (tile_p1)
     int mt0;     // first M-tile
     int mts;     // number of M-tiles (accumulators) in this item
 };
@@ -91,6 +91,7 @@ struct TcParams {
     int kind;                      // TC_TF32 / TC_BF16X3 / TC_BF16X2 / TC_FP64E
     int kcs_max;                   // largest p2 chunk count of the launch (rank variant)
     unsigned long long wait_ns;    // limit of each wait (kWaitNs if 0)
+    int split;                     // p1 values per M-tile: 128 / n3 / split (tile_p1)
     int withhold;                  // test aid: CTA 0 issues only withhold - 1 integral loads (0 = off)
 };
 
@@ -344,7 +345,7 @@ __device__ __forceinline__ unsigned short to_bf16_bits(float x)
     return __bfloat16_as_ushort(__float2bfloat16_rn(x));
 }
 
-// Geometry of the current item, derived from its descriptor.
+// Geometry of an item, derived from its descriptor.
 struct ItemGeo {
     int n0, n1, n2, n3;
     int o0, o2;
@@ -355,8 +356,14 @@ struct ItemGeo {
     int rows;         // n1 * n3
 };
 
-__device__ __forceinline__ ItemGeo geo_of(const DimerDesc& d, int f, int p1t)
+// The FP64E kernel, at its register limit, forms the p1 values per M-tile from the
+// launch's split: read from the item they cost its first half 1.4 % (2216 dimers of
+// 32 AO 16.20 -> 16.46 ms; formed 16.28), while the other kernels are a little
+// faster for reading them (BF16x2, 1036 dimers: 2.637 ms against 2.649).
+template <int KIND>
+__device__ __forceinline__ ItemGeo geo_of(const DimerDesc& d, const TcItem& item, int split)
 {
+    const int f = item.form;
     ItemGeo g;
     g.n0 = d.nX;
     g.n1 = f ? d.nY : d.nX;
@@ -364,7 +371,8 @@ __device__ __forceinline__ ItemGeo geo_of(const DimerDesc& d, int f, int p1t)
     g.n3 = f ? d.nX : d.nY;
     g.o0 = d.oX;
     g.o2 = d.oY;
-    g.p1t = p1t;
+    if constexpr (KIND == TC_FP64E) g.p1t = split > 1 ? max(1, 128 / g.n3 / split) : 128 / g.n3;
+    else g.p1t = item.p1t;
     g.kcs = (g.n2 + kKC - 1) / kKC;
     g.kblocks = g.n0 * g.kcs;
     g.N = d.npad;
@@ -462,7 +470,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_half_tc(const TcParams P)
             for (int it = blockIdx.x; it < P.n_items && !sh->abort; it += gridDim.x) {
                 const TcItem item = P.items[it];
                 const DimerDesc& d = P.desc[item.dimer];
-                const ItemGeo g = geo_of(d, item.form, item.p1t);
+                const ItemGeo g = geo_of<KIND>(d, item, P.split);
                 const CUtensorMap* map = P.maps + 2 * item.dimer + item.form;
                 const unsigned box = (unsigned)g.n3 * kKC * g.p1t * 8u;
                 for (int kb = 0; kb < g.kblocks && !sh->abort; kb++) {
@@ -493,7 +501,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_half_tc(const TcParams P)
             bool any = false;
             for (int it = blockIdx.x; it < P.n_items && !sh->abort; it += gridDim.x, li++) {
                 const TcItem item = P.items[it];
-                const ItemGeo g = geo_of(P.desc[item.dimer], item.form, item.p1t);
+                const ItemGeo g = geo_of<KIND>(P.desc[item.dimer], item, P.split);
                 const unsigned idesc = make_idesc(KIND, g.N);
                 const int b = li & 1;
                 if (!mbar_wait(&sh->tmem_empty[b], ((li >> 1) & 1) ^ 1, &sh->abort, P.status, 2, P.wait_ns)) break;
@@ -545,7 +553,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_half_tc(const TcParams P)
         for (int it = blockIdx.x; it < P.n_items && !sh->abort; it += gridDim.x) {
             const TcItem item = P.items[it];
             const DimerDesc& d = P.desc[item.dimer];
-            const ItemGeo g = geo_of(d, item.form, item.p1t);
+            const ItemGeo g = geo_of<KIND>(d, item, P.split);
             const float* CX = P.Cf + d.cX;
             const float* CY = P.Cf + d.cY;
             const int npairs = g.o0 * g.o2;
@@ -668,7 +676,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_half_tc(const TcParams P)
         for (int it = blockIdx.x; it < P.n_items && !sh->abort; it += gridDim.x, li++) {
             const TcItem item = P.items[it];
             const DimerDesc& d = P.desc[item.dimer];
-            const ItemGeo g = geo_of(d, item.form, item.p1t);
+            const ItemGeo g = geo_of<KIND>(d, item, P.split);
             const int b = li & 1;
             if (!mbar_wait(&sh->tmem_full[b], (li >> 1) & 1, &sh->abort, P.status, 8, P.wait_ns)) break;
             tc_fence_after();
@@ -1426,7 +1434,7 @@ __global__ void __launch_bounds__(rank_threads<BIG, OB, KIND>(), 1) k_half_tc_ra
             bool ok = true;
             for (int it = blockIdx.x; it < P.n_items && ok && !*abort; it += gridDim.x) {
                 const TcItem item = P.items[it];
-                const ItemGeo g = geo_of(P.desc[item.dimer], item.form, item.p1t);
+                const ItemGeo g = geo_of<KIND>(P.desc[item.dimer], item, P.split);
                 const CUtensorMap* map = P.maps + 2 * item.dimer + item.form;
                 const unsigned box = (unsigned)g.n3 * kKC * g.p1t * 8u;
                 for (int mt = 0; mt < item.mts && ok; mt++)
@@ -1466,7 +1474,7 @@ __global__ void __launch_bounds__(rank_threads<BIG, OB, KIND>(), 1) k_half_tc_ra
             for (int u = 0; u < 6; u++) idesc_f6[u] = make_idesc(KIND, (7 - u) * kNT);
             for (int it = blockIdx.x; it < P.n_items && ok && !*abort; it += gridDim.x, li++) {
                 const TcItem item = P.items[it];
-                const ItemGeo g = geo_of(P.desc[item.dimer], item.form, item.p1t);
+                const ItemGeo g = geo_of<KIND>(P.desc[item.dimer], item, P.split);
                 const int wp = li & 1;
                 if (!(ok = mbar_wait(&sh->full_w[wp], (li >> 1) & 1, abort, P.status, 12, P.wait_ns))) break;
                 for (int mt = 0; mt < item.mts && ok; mt++)
@@ -1571,7 +1579,7 @@ __global__ void __launch_bounds__(rank_threads<BIG, OB, KIND>(), 1) k_half_tc_ra
         for (int it = blockIdx.x; it < P.n_items && ok && !*abort; it += gridDim.x, li++) {
             const TcItem item = P.items[it];
             const DimerDesc& d = P.desc[item.dimer];
-            const ItemGeo g = geo_of(d, item.form, item.p1t);
+            const ItemGeo g = geo_of<KIND>(d, item, P.split);
             const float* CY = P.Cf + d.cY;
             [[maybe_unused]] const double* CYd = P.Cd + d.cY;   // FP64E: C_Y in FP64
             const int wp = li & 1;
@@ -1765,7 +1773,7 @@ __global__ void __launch_bounds__(rank_threads<BIG, OB, KIND>(), 1) k_half_tc_ra
         for (int it = blockIdx.x; it < P.n_items && ok && !*abort; it += gridDim.x, li++) {
             const TcItem item = P.items[it];
             const DimerDesc& d = P.desc[item.dimer];
-            const ItemGeo g = geo_of(d, item.form, item.p1t);
+            const ItemGeo g = geo_of<KIND>(d, item, P.split);
             const int par = li & 1;
             float* cx = cxs + par * CXF;
             // stage C_X's occupied columns, row p0 = e, for this item
@@ -2178,8 +2186,8 @@ cudaError_t tc_prepare(TcKind kind, const DimerDesc* h_desc, const DimerDesc* d_
             for (int q = 0; q < nit; q++) {
                 TcItem it;
                 it.dimer = k;
-                it.form = f;
-                it.p1t = p1t;
+                it.form = (short)f;
+                it.p1t = (short)p1t;
                 it.mt0 = q * mmax;
                 it.mts = std::min(mmax, tiles - it.mt0);
                 items.push_back(it);
@@ -2215,6 +2223,7 @@ cudaError_t tc_prepare(TcKind kind, const DimerDesc* h_desc, const DimerDesc* d_
     TcLaunch& P = *out;
     P.items = w + items_off;
     P.n_items = (int)items.size();
+    P.split = split;
     P.maps = w;
     P.desc = d_desc;
     P.Cf = Cf;
@@ -2263,6 +2272,7 @@ cudaError_t tc_launch(const TcLaunch& L, cudaStream_t s)
     TcParams P;
     P.items = static_cast<const TcItem*>(L.items);
     P.n_items = L.n_items;
+    P.split = L.split;
     P.maps = static_cast<const CUtensorMap*>(L.maps);
     P.desc = L.desc;
     P.Cf = L.Cf;
