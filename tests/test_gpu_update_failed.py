@@ -56,3 +56,45 @@ def test_packed_update_at_the_cap():
                     assert np.array_equal(x, y)
     # three caps a buffer: some that refuse the first, some that refuse the second only
     assert refused >= 4
+
+
+def test_packed_update_of_borrowed_dimers_at_the_cap():
+    """The dimers' own storage, which an update of borrowed ones needs, refused
+    for the first, some or the last of them: they stay borrowed.  (The plan is
+    rebuilt by moving one dimer to a copy of its integrals.)"""
+    torch = pytest.importorskip("torch")
+    rng = np.random.default_rng(20)
+    A, K, CX, eX, CY, eY = rand_dimer(rng, NX, NY, 2, 3)
+    nd = 8
+    p = np.tile(synth.pack_blocks(A, K), nd)
+    offsets = np.arange(nd, dtype=np.uint64) * (p.size // nd)
+    block = 2 * 8 * (NX * NY) ** 2
+    buf = torch.from_numpy(np.concatenate([A.ravel(), K.ravel()])).cuda()
+    twin = buf.clone()
+    torch.cuda.synchronize()
+    refused = done = 0
+    cap = block
+    while done < 2:
+        assert refused < 100
+        with M.Context(precision="fp64", mem_cap_bytes=cap, validate=False) as ctx:
+            cap += block // 3
+            try:
+                for d in range(nd):
+                    X, Y = ctx.add_monomer(CX, eX, 2), ctx.add_monomer(CY, eY, 3)
+                    ctx.add_dimer(X, Y, buf.data_ptr(), M.MCPT_AO_BLOCKS, on_device=1)
+                ctx.run()
+            except M.McptError as e:
+                assert e.status == M.MCPT_ENOMEM
+                continue
+            before = ctx.energies()[2].copy()
+            try:
+                ctx.update_dimers(0, nd, 2.0 * p, offsets, M.MCPT_AO_PACKED)
+                done += 1
+            except M.McptError as e:
+                assert e.status == M.MCPT_ENOMEM
+                refused += 1
+                assert np.array_equal(ctx.energies()[2], before)
+                ctx.update_dimer(nd - 1, twin.data_ptr(), M.MCPT_AO_BLOCKS, on_device=1)
+                ctx.run()
+                assert np.array_equal(ctx.energies()[2], before)
+    assert refused >= 2 * nd
