@@ -262,8 +262,8 @@ struct DfMax {
 void df_smem_elems(int nX, int nY, int oX, int oY, int* u_elems, int* c_elems);
 long long df_half_elems(bool fp64, int naux, int nX, int nY, int oX, int oY);
 // Terms of nd dimers into E2 (2 doubles each): FP64 arithmetic if fp64,
-// else FP32 (energy epilogue on FP32 pairs, FP64 sums).  half: scratch of the
-// half-transformed blocks; part: 2 doubles per occupied pair.
+// else FP32 (energy epilogue FP64).  half: scratch of the half-transformed
+// blocks; part: 2 doubles per occupied pair.
 cudaError_t launch_df(bool fp64, const DfDim* dims, int nd, const DfMax& m, const double* C, const double* eps,
                       void* half, double* part, double* E2, int sms, cudaStream_t s);
 

@@ -249,11 +249,12 @@ __device__ __forceinline__ void df_term(double& sj, double& sk, float v, float w
 
 // The j block [j0, j0 + JB) of occupied i: a thread holds 4 a x 4 b x JB values of
 // (ia|jb) and of (ib|ja), two per packed multiply-add; per Q, 2 + 2 JB 16-byte
-// shared loads feed 32 JB multiply-adds.  Bound by shared-memory bandwidth and
-// the FP32 pipes.  The kernel before it took one (i, j) per CTA with one
-// element per thread (4 shared loads per 2 multiply-adds) and an FP64 division
-// per term (0.5 ms of FP64 pipe): 2.08 ms for 1036 dimers of 32 + 32 AO and
-// naux 192 against 0.55 ms.
+// shared loads feed 32 JB multiply-adds.  Bound by latency at two warps per
+// scheduler (231 registers; FMA pipe 32 % busy, shared memory 23 % of its
+// wavefronts), then by the FP64 pipe in the epilogue.  The kernel before it took
+// one (i, j) per CTA with one element per thread (4 shared loads per 2
+// multiply-adds) and an FP64 division per term: 2.08 ms for 1036 dimers of
+// 32 + 32 AO and naux 192 against 0.75 ms (0.24 of it the epilogue).
 template <int JB>
 __device__ __forceinline__ void df_pairs(const DfDim& d, const double* __restrict__ eps,
                                          const float* __restrict__ half, int i, int j0, float* buf, double& ej,

@@ -20,10 +20,12 @@
 // no FP64 operation per term.  The FP64-pipe variant of that epilogue (five
 // FP64 operations per term) stays selectable for comparison.
 // Monomers of at most 32 AO: one warp per occupied pair, a dimer's pairs over
-// one or more CTAs.
-// Larger ones: register-tiled GEMMs, one CTA per range of a dimer's pairs,
-// the ranges' partial sums added per dimer in range order.  Every sum has a
-// fixed order: the energies are deterministic run to run, with no atomics.
+// one or more CTAs; the last of them to arrive adds the pairs' sums.
+// Larger ones: register-tiled GEMMs, one CTA per range of a dimer's pairs; one
+// partial sum per range in FP64, one per pair in FP32, added per dimer with
+// strided lanes and a fixed tree.  Every sum has a fixed order, so the energies
+// are deterministic run to run: the only atomics are arrival counters (zero
+// before a launch and after it) that pick the block which does the last pass.
 #include "internal.h"
 #include "convert.h"
 #include "ff.h"

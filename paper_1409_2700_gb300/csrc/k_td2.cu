@@ -369,8 +369,9 @@ k_pgemm_dw(const PGemm<T>* __restrict__ tabs)
 constexpr int kFR = 48, kFC = 48, kFK = 32, kFThreads = 96;
 constexpr int kFS = kFR + 6;                   // row stride of the staged [k][r], [k][c] (8-byte rows; 2-way transposed stores)
 
-// Offsets fit 32 bits: an operand spans at most the n_X^2 n_Y^2 <= 128^4
-// elements of a dimer's block.
+// Offsets fit 32 bits for monomers of at most 128 AO: an operand is the dimer's
+// n_X^2 n_Y^2 <= 2^28 integrals, the packed ladder matrix (fewer), a monomer's
+// (o v)^2 or the dimer's o_X v_X o_Y v_Y (o v <= 64^2: at most 2^24).
 __device__ __forceinline__ int ax_off32(const PAxis& a, int x)
 {
     return (x / a.n1) * (int)a.s0 + (x % a.n1) * (int)a.s1;
